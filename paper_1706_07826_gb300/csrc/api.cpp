@@ -447,7 +447,14 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
                 const int ns = pm1_nslot(P, Q, blk);
                 if (ns > 0 && pm1_shape_ok(blk, ns, md, 0)) { sh = SweepShape{1, blk, Q, 0, ns, md}; break; }
             }
-        // large problems: the streaming kernel (one quad per CTA)
+        // large problems: the quad-group kernel, or (large biases) the streaming one (one quad per CTA)
+        if (sh.kind == 0 && pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
+            SweepShape c = pm1q_default(H.n, md, (size_t)optin);
+            if (c.block > 0) {
+                c.Q = pm1q_sample_quads(quads, sms, c.Q, pm1q_layout(c.block, H.n, c.Q, md).nv);
+                sh = c;
+            }
+        }
         if (sh.kind == 0 && pm1s_shape_ok(512, md, H.n, 1) &&
             pm1s_smem_bytes(H.n, 1, md) <= (size_t)optin)
             sh = SweepShape{2, 512, 1, 0, 0, md};

@@ -316,19 +316,38 @@ __global__ void __launch_bounds__(256) k_slots_init(Slot *slots, SolveConsts C)
 }
 
 // Quads per work item of a start whose current problem is P and who runs
-// nquads quads: C.Q; for the quad-group kernel the most that the launch's
-// shared memory holds; for the register kernel the most that its slots hold
+// nquads quads: C.Q; for the quad-group kernel see below; for the register
+// kernel the most that its slots hold
 // (every colour class fills ceil(size * q / block) whole slots; at most
 // block * nslot / 4 quads so that the per-item energy sums fit), but no more
 // than leaves about two items per CTA of the launch (starts of similar size).
-__device__ __forceinline__ int item_quads(const DevProb *P, const SolveConsts &C, int nquads)
+// Quad-group kernel: the size, up to 64 quads and what the launch's shared memory
+// holds, that finishes first when SMs take equal shares of the launch (`load`: spins
+// times quads of every start): one item's length where no SM gets two (`quads`: those
+// of every start), else the shares and half an item for the last one.  An item costs a
+// fixed part and each of its groups; one lone quad costs three fifths of a pair.
+__device__ __forceinline__ int item_quads(const DevProb *P, const SolveConsts &C, int nquads, long long load,
+                                          long long quads)
 {
-    const int cap = max(1, (int)(((long long)nquads * C.nslots) / (2ll * max(C.grid, 1))));
     if (C.fit_words > 0) {
-        // quad-group kernel: as many quads as the launch's spin words hold, at most 64
-        const int fit = C.fit_words / (2 * (P->n + 1));
-        return max(1, min(min(fit, 64), cap));
+        const int fit = min(64, max(1, 2 * pm1q_fit_pairs(C.fit_words, P->n, C.fit_rec, C.fit_nv)));
+        const int step = 2 * C.fit_nv, per = C.fit_nv == 1 ? 4 : 7;
+        const float share = (float)load / ((float)max(P->n, 1) * (float)C.sms);  // quads of this size per SM
+        int best = 1;
+        float best_t = 3e38f;
+        for (int q = C.fit_nv == 1 ? 1 : step; q <= max(fit, step) && q < nquads + step; q += q == 1 ? 1 : step) {
+            const float cost = q == 1 ? 3.f : (float)(per * ceil_div(q, step) + 1);
+            const float t = quads <= (long long)C.sms * q ? cost : cost * (share / (float)q + 0.5f);
+            if (t < best_t) {
+                best_t = t;
+                best = q;
+            }
+        }
+        if (best <= step) return max(1, min(best, fit));
+        const int even = ceil_div(nquads, ceil_div(nquads, best));
+        return min(best, ceil_div(even, step) * step);
     }
+    const int cap = max(1, (int)(((long long)nquads * C.nslots) / (2ll * max(C.grid, 1))));
     if (C.fit_block <= 0) return C.Q;
     const int ncol = P->ncol;
     auto need = [&](int q) {
@@ -356,8 +375,21 @@ __global__ void __launch_bounds__(kBigBlock)
 {
     __shared__ int s_warp[32];
     __shared__ int s_off[kBigBlock], s_groups[kBigBlock], s_qn[kBigBlock], s_nquads[kBigBlock];
+    __shared__ unsigned long long s_load, s_quads;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int carry = 0;
+    if (C.fit_words > 0) {
+        if (threadIdx.x == 0) s_load = s_quads = 0;
+        __syncthreads();
+        for (int si = threadIdx.x; si < C.nslots; si += blockDim.x) {
+            const Slot &s = slots[si];
+            if (s.mode == kDone) continue;
+            const unsigned long long q = (unsigned long long)ceil_div(phase_samples(C, s.mode), 4);
+            atomicAdd(&s_load, q * (unsigned long long)s.cur->n);
+            atomicAdd(&s_quads, q);
+        }
+        __syncthreads();
+    }
     for (int base = 0; base < C.nslots; base += blockDim.x) {
         const int si = base + threadIdx.x;
         int groups = 0, qn = 1, nquads = 0;
@@ -383,7 +415,7 @@ __global__ void __launch_bounds__(kBigBlock)
                 j.t1 = t1;
                 jobs[si] = j;
                 nquads = ceil_div(S, 4);
-                qn = item_quads(s.cur, C, nquads);
+                qn = item_quads(s.cur, C, nquads, (long long)s_load, (long long)s_quads);
                 groups = ceil_div(nquads, qn);
                 if (t0 == 0) {
                     s.rec_count[s.phase] = S;

@@ -39,7 +39,12 @@ cudaError_t engine_phase(const PhaseEngine &E, Slot *slots, int nslots, int T, i
     C.Q = E.shape.Q;
     C.fit_block = E.shape.kind == 1 ? E.shape.block : 0;
     C.fit_nslot = E.shape.kind == 1 ? E.shape.nslot : 0;
-    C.fit_words = E.shape.kind == 6 ? 2 * E.shape.Q * (E.max_n0 + 1) : 0;
+    QuadLayout ql{1, 0, 0, 0, 0};
+    if (E.shape.kind == 6) ql = pm1q_layout(E.shape.block, E.max_n0, E.shape.Q, E.shape.maxd);
+    C.fit_words = ql.fit_words;
+    C.fit_rec = ql.rec;
+    C.fit_nv = ql.nv;
+    C.sms = E.sms;
     C.grid = grid;
     C.T = T;
     cudaError_t e = launch_plan(slots, C, E.jobs, E.items, E.ctr + 0, E.ctr + 1, E.ctr + 2, st);
@@ -214,7 +219,7 @@ void solve_cache_put(std::vector<int64_t> key, spvar_plan *pl)
 
 int grid_for(const spvar_plan *pl, int items)
 {
-    const int occ = std::max(1, sweep_shape_occupancy(pl->shape, pl->pm1, pl->sweep_smem));
+    const int occ = std::max(1, sweep_shape_occupancy(pl->shape, pl->pm1, pl->max_n0, pl->sweep_smem));
     const int full = occ * pl->sms;
     if (!pl->shape.balance || items <= full) return std::max(1, std::min(items, full));
     return ceil_div(items, ceil_div(items, full));
@@ -228,6 +233,7 @@ PhaseEngine engine_of(const spvar_plan *pl)
     E.pm1 = pl->pm1;
     E.max_n0 = pl->max_n0;
     E.max_deg = pl->max_deg;
+    E.sms = pl->sms;
     E.thr_stride = pl->thr_stride;
     E.thr = pl->d_thr;
     E.ent = pl->d_ent;
@@ -373,23 +379,30 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
         }
         return out;
     }
-    if (pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
+    // +-1 couplers and dmax <= 30: the quad-group and the register kernel.  The streaming, the
+    // warp-per-quad and the general kernel lost to the quad-group kernel at every size measured
+    // (3D L = 9, 20 starts x (250 + 250): 6.4 ms against 9.3 ms warp per quad and 13.2 ms
+    // streaming; L = 12: 10.8 against 14.0 streaming; the uneven batch of L = 6 .. 12: 37 against
+    // 104), so they are tried only where it does not apply.
+    const bool quads_ok = pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg);
+    const size_t listed = out.size();
+    if (quads_ok) {
+        const int md = pl->max_deg <= 6 ? 6 : 8;
+        const int shapes[][2] = {{128, 2}, {128, 4}, {256, 2}, {256, 4}, {256, 8}, {512, 2}, {512, 4}, {512, 8}, {1024, 2}, {1024, 16}};
+        for (const auto &bq : shapes) {
+            SweepShape sh{6, bq[0], bq[1], 0, 0, md};
+            if (pm1q_shape_ok(bq[0], md, pl->max_n0, bq[1]) &&
+                sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
+                out.push_back(sh);
+        }
+    }
+    const bool others = out.size() == listed;
+    if (others && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
         const int md = pl->max_deg <= 6 ? 6 : 8;
         for (int w : {2, 4, 8, 16})
             for (int K : {2, 4}) {
                 SweepShape sh{4, 32 * w, w, 0, K, md};
                 if (pm1w_shape_ok(w, md, pl->max_n0, K) &&
-                    sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
-                    out.push_back(sh);
-            }
-    }
-    if (pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
-        // quad-group kernel: Q quads of the largest problem per item (more for smaller ones)
-        const int md = pl->max_deg <= 6 ? 6 : 8;
-        for (int b : {128, 256, 512})
-            for (int Q : {1, 2, 4, 8}) {
-                SweepShape sh{6, b, Q, 0, 0, md};
-                if (pm1q_shape_ok(b, md, pl->max_n0, Q) &&
                     sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
                     out.push_back(sh);
             }
@@ -401,11 +414,11 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
         for (int qi = 0; qi < 4; ++qi) {
             const int Q = qs[qi];
             if (Q > 1 && quads < Q) continue;
-            for (int stg = 1; stg >= 0; --stg) {
+            for (int stg = 1; others && stg >= 0; --stg) {
                 SweepShape sh{0, blocks[bi], Q, stg, 0, 0};
                 if (sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin) out.push_back(sh);
             }
-            if (Q == 1 && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
+            if (others && Q == 1 && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
                 const int md = pl->max_deg <= 6 ? 6 : 8;
                 for (int sb : {128, 256, 512, 1024}) {
                     if (sb != blocks[bi] && !(bi == 2 && sb == 1024)) continue;
@@ -484,7 +497,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
     auto trial = [&](const SweepShape &sh, int chunk_t) -> float {
         pl->shape = sh;
         pl->sweep_smem = sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg);
-        if (sweep_shape_occupancy(sh, pl->pm1, pl->sweep_smem) < 1) return 1e30f;
+        if (sweep_shape_occupancy(sh, pl->pm1, pl->max_n0, pl->sweep_smem) < 1) return 1e30f;
         const int nslots = (pl->prm.form == SPVAR_FORM_PLAIN) ? 1 : pl->C.nslots;
         pl->C.Q = sh.Q;
         pl->C.chunk = chunk_t;
@@ -863,7 +876,8 @@ int spvar_plan_create(const spvar_problem *const *problems, int32_t nproblems,
             }
         } else if (p.sweep_kernel == SPVAR_SWEEP_PM1Q) {
             const int md = pl->max_deg <= 6 ? 6 : 8;
-            if (!pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg) || !pm1q_shape_ok(blk, md, pl->max_n0, Q)) {
+            if (!pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg) || !pm1q_shape_ok(blk, md, pl->max_n0, Q) ||
+                !pm1q_request_ok(pl->max_n0, Q, (size_t)optin)) {
                 plan_free(pl);
                 return SPVAR_ELIMIT;
             }

@@ -503,14 +503,11 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
     const int blk = p.sweep_block ? p.sweep_block : 512;
     E.shape = SweepShape{0, blk, Q, 1, 0, 0};
     if (sweep_shape_smem(E.shape, cfg->max_n, stride, cfg->max_degree) > (size_t)optin) E.shape.stage = 0;
-    // +-1-only servers: the streaming +-1 kernel (one quad per CTA, per-spin data
-    // staged once per CTA), or with SPVAR_SWEEP_PM1Q the quad-group +-1 kernel
-    // (work items of Q quads of the largest admissible problem, more quads of
-    // smaller ones).  Measured at a request's 20 starts x 250 samples of 3D +-J
-    // problems, the streaming kernel leads at every size (L = 8: 3.3e11 against
-    // 2.7e11 attempts/s; L = 12: 6.3e11 against 4.8e11; L = 20: 6.9e11 against
-    // 4.0e11): the quad-group kernel pays off only when a problem has hundreds of
-    // quads to group.
+    // +-1-only servers: the quad-group +-1 kernel where dmax <= 30 (with SPVAR_SWEEP_PM1Q in
+    // items of Q quads of the largest admissible problem, more of smaller ones), else the
+    // streaming +-1 kernel.  Measured at a request's 20 starts x (250 + 250) samples of 3D +-J
+    // problems, quad-group against streaming: L = 9 6.4 against 13.2 ms, L = 12 10.8 against
+    // 14.0, L = 20 18.7 against 23.8.
     const int md = cfg->max_degree <= 6 ? 6 : 8;
     const bool pm1_only = p.sweep_kernel == SPVAR_SWEEP_PM1 || p.sweep_kernel == SPVAR_SWEEP_PM1S ||
                           p.sweep_kernel == SPVAR_SWEEP_PM1Q;
@@ -519,10 +516,18 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
     if (pm1_only && want_quads && cfg->max_degree <= 8 && cfg->max_dmax <= 30) {
         const int qb = (p.sweep_block == 128 || p.sweep_block == 256) ? p.sweep_block : 512;
         SweepShape sh{6, qb, Q, 0, 0, md};
-        if (pm1q_shape_ok(qb, md, cfg->max_n, Q) && sweep_shape_smem(sh, cfg->max_n, stride, cfg->max_degree) <= (size_t)optin) {
+        if (pm1q_shape_ok(qb, md, cfg->max_n, Q) && pm1q_request_ok(cfg->max_n, Q, (size_t)optin)) {
             E.shape = sh;
             chosen = true;
         }
+    }
+    const bool auto_quads = !chosen && p.sweep_kernel == SPVAR_SWEEP_PM1 && p.sweep_block == 0 &&
+                            p.replicas_per_block == 0 && cfg->max_degree <= 8 && cfg->max_dmax <= 30 &&
+                            pm1q_default(cfg->max_n, md, (size_t)optin).block > 0;
+    if (auto_quads) {
+        E.shape = pm1q_default(cfg->max_n, md, (size_t)optin);
+        Q = E.shape.Q;
+        chosen = true;
     }
     if (!chosen && pm1_only && cfg->max_degree <= 8 && cfg->max_dmax <= 254 && pm1s_shape_ok(blk, md, cfg->max_n, 1)) {
         SweepShape sh{2, blk, 1, 0, 0, md};
@@ -555,6 +560,7 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
     E.pm1 = pm1_only;
     E.max_n0 = cfg->max_n;
     E.max_deg = cfg->max_degree;
+    E.sms = S->sms;
     E.thr_stride = stride;
     E.thr = (const uint32_t *)(w + o_thr);
     E.jobs = (SweepJob *)(w + o_jobs);
@@ -580,8 +586,12 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
         t.E = E;
         t.E.max_n0 = tn;
         t.E.C.max_n0 = tn;
-        t.E.sweep_smem = sweep_shape_smem(E.shape, tn, stride, cfg->max_degree);
-        const int occ = std::max(1, sweep_shape_occupancy(t.E.shape, t.E.pm1, t.E.sweep_smem));
+        if (auto_quads && !sqa) {
+            t.E.shape = pm1q_default(tn, md, (size_t)optin);
+            t.E.C.Q = t.E.shape.Q;
+        }
+        t.E.sweep_smem = sweep_shape_smem(t.E.shape, tn, stride, cfg->max_degree);
+        const int occ = std::max(1, sweep_shape_occupancy(t.E.shape, t.E.pm1, tn, t.E.sweep_smem));
         t.grid = occ * S->sms;
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(S->cap_st, cudaStreamCaptureModeRelaxed) == cudaSuccess) {

@@ -17,6 +17,8 @@ constexpr int kMaxColours = SPVAR_MAX_DEGREE + 1;
 constexpr uint32_t kSweepBits = 20;                 // counter word 1 = phase << 20 | sweep
 constexpr uint32_t kInitSlot = (1u << kSweepBits) - 1u;
 
+__host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
 // Device-resident problem: CSR in index order plus the sweep layout.
 // "Positions" order the spins colour class by colour class, increasing index
 // inside a class; the sweep kernels work in positions so that one colour is
@@ -154,14 +156,16 @@ struct SolveConsts {
     // register kernel: work items take as many quads as the slots hold (block
     // threads x nslot items per thread, colour classes in whole slots); 0: Q quads
     int32_t fit_block, fit_nslot, grid;  // grid: CTAs of the sweep launch
-    int32_t fit_words;                   // quad-group kernel: spin words of the launch's shared memory
+    // quad-group kernel: words of the launch's shared memory for records and groups (0: another kernel), words
+    // of a spin's record, pairs of quads per group, SMs
+    int32_t fit_words, fit_rec, fit_nv, sms;
     // sweeps per phase, and sweeps per launch (0: the whole phase in one launch).  With
     // chunk > 0 a phase's sample is annealed over ceil(T / chunk) launches, each resuming
     // from the states the previous one wrote; the persistence pass runs after the last.
     int32_t T, chunk;
     // PTICM as the sampler: a phase's sample size is the number of states its run
     // kept (the slot's rec_count of the phase), and the elite is ceil(elite x that)
-    int32_t pticm, pad2;
+    int32_t pticm;
     double elite;
 };
 // Elite count k = ceil(elite * S), clamped to [1, S] (host and device).
@@ -235,7 +239,6 @@ inline void fill_solve_consts(const spvar_params &p, SolveConsts &C)
     C.T = p.num_sweeps;
     C.chunk = 0;
     C.pticm = p.sampler == SPVAR_SAMPLER_PTICM ? 1 : 0;
-    C.pad2 = 0;
     C.elite = p.elite_threshold;
 }
 // Sweep launches per phase: ceil(T / chunk), or 1 without chunking.
@@ -349,12 +352,51 @@ inline int sqa_reg_ncls(int ncol, int max_class, int block, int P)
     return ncol <= 2 ? 2 : 4;
 }
 
+// Launch shape of a sweep: kind 0 = general kernel (stage: layout staged in
+// shared memory), kind 1 = register-resident kernel (nslot items per thread,
+// maxd neighbour registers per item; stage = 1: the 16-bit-lane variant for
+// one coupler magnitude per spin, stage = 2: its variant for small integer
+// couplers), kind 2 = streaming +-1 kernel
+// (maxd neighbour offsets per spin staged in shared memory, Q = 1), kind 4 =
+// warp-per-quad +-1 kernel (Q = warps = block / 32; nslot = spins in flight per lane,
+// 2 or 4), kind 5 = simulated
+// quantum annealing (Q = 1).  A persistent grid holds
+// every CTA the SMs can keep resident, or (balance) the fewest CTAs that still
+// need the same number of waves of items, so that no last wave runs nearly empty.
+struct SweepShape {
+    int kind, block, Q, stage, nslot, maxd;
+    int balance = 0;  // 1: grid sized so that every CTA runs the same number of items
+    int slices = 0;   // kind 5 (SQA): Trotter slices; stage = the variant (0 general, 1 +-1 walk,
+                      // 2 +-1 register form), nslot the acceptance-table width W, maxd the largest degree
+    int ncls = 0;     // kind 5, variant 2: colour-class slots per thread (2 or 4)
+    int ent32 = 0;    // kind 5, variant 2: 32-bit acceptance entries (no entry of the table is 2^32)
+    int lpp = 1;      // sweep launches per phase (the autotuner's sweeps-per-launch axis)
+};
 // Quad-group +-1 sweep (sweep_pm1q.cu): up to 64 quads of one problem per work
 // item, spin words only in shared memory (2 (n + 1) words per quad).
+// Shared-memory words of one group of nv pairs of quads: 12 of Philox products per pair, two
+// copies of the spin words and their closing zero words, rounded up to 16 bytes.
+constexpr int kPairHead = 12;
+__host__ __device__ inline int group_words(int n, int nv) { return (nv * (kPairHead + 2 * (n + 1)) + 3) & ~3; }
+// Pairs an n-spin problem gets in `words` words beside its records of `rec` words a spin.
+__host__ __device__ inline int pm1q_fit_pairs(int words, int n, int rec, int nv)
+{
+    return nv * ((words - ((rec * n + 3) & ~3)) / group_words(n, nv));
+}
+constexpr int kUnitRows = 8;  // rounds of the block whose units are listed in shared memory (with records)
 bool pm1q_shape_ok(int block, int maxd, int max_n, int Q);
-size_t pm1q_smem_bytes(int max_n, int Q);
-cudaError_t launch_sweep_pm1q(const SweepLaunch &L, int block, int maxd, int grid, size_t smem, cudaStream_t st);
-int pm1q_max_active_blocks(int block, int maxd, size_t smem);
+struct QuadLayout {
+    int nv, rec, unit_rows;  // pairs of quads per group, words of a spin's record (0: none), listed rounds of units
+    int fit_words;           // words for records and groups
+    size_t bytes;            // dynamic shared memory
+};
+QuadLayout pm1q_layout(int block, int max_n, int Q, int maxd);
+SweepShape pm1q_default(int max_n, int maxd, size_t optin);
+int pm1q_sample_quads(int quads, int sms, int Q, int nv);
+// A requested item of Q quads is taken where two copies of every quad's spin words fit a CTA.
+inline bool pm1q_request_ok(int max_n, int Q, size_t optin) { return 8 * (size_t)Q * ((size_t)max_n + 1) <= optin; }
+cudaError_t launch_sweep_pm1q(const SweepLaunch &L, int block, int maxd, int Q, int grid, size_t smem, cudaStream_t st);
+int pm1q_max_active_blocks(int block, int maxd, int max_n, int Q, size_t smem);
 
 // PTICM sampler (sweep_pticm.cu): one CTA per run, every replica's spins in
 // shared memory.
@@ -382,26 +424,6 @@ cudaError_t launch_sweep_pm1w(const SweepLaunch &L, int warps, int maxd, int K, 
                               cudaStream_t st);
 int pm1w_max_active_blocks(int warps, int maxd, int K, size_t smem);
 
-// Launch shape of a sweep: kind 0 = general kernel (stage: layout staged in
-// shared memory), kind 1 = register-resident kernel (nslot items per thread,
-// maxd neighbour registers per item; stage = 1: the 16-bit-lane variant for
-// one coupler magnitude per spin, stage = 2: its variant for small integer
-// couplers), kind 2 = streaming +-1 kernel
-// (maxd neighbour offsets per spin staged in shared memory, Q = 1), kind 4 =
-// warp-per-quad +-1 kernel (Q = warps = block / 32; nslot = spins in flight per lane,
-// 2 or 4), kind 5 = simulated
-// quantum annealing (Q = 1).  A persistent grid holds
-// every CTA the SMs can keep resident, or (balance) the fewest CTAs that still
-// need the same number of waves of items, so that no last wave runs nearly empty.
-struct SweepShape {
-    int kind, block, Q, stage, nslot, maxd;
-    int balance = 0;  // 1: grid sized so that every CTA runs the same number of items
-    int slices = 0;   // kind 5 (SQA): Trotter slices; stage = the variant (0 general, 1 +-1 walk,
-                      // 2 +-1 register form), nslot the acceptance-table width W, maxd the largest degree
-    int ncls = 0;     // kind 5, variant 2: colour-class slots per thread (2 or 4)
-    int ent32 = 0;    // kind 5, variant 2: 32-bit acceptance entries (no entry of the table is 2^32)
-    int lpp = 1;      // sweep launches per phase (the autotuner's sweeps-per-launch axis)
-};
 // The streaming and warp-per-quad kernels apply to +-1 couplers, degree <= 8
 // and dmax <= 254; the register kernel needs dmax <= 30.
 inline bool pm1_kernel_eligible(bool pm1, int dmax, int maxdeg) { return pm1 && dmax <= 254 && maxdeg <= 8; }
@@ -430,7 +452,7 @@ inline size_t sweep_shape_smem(const SweepShape &s, int max_n, int thr_stride, i
     if (s.kind == 1) return pm1_smem_bytes(s.stage != 0, thr_stride);
     if (s.kind == 2) return pm1s_smem_bytes(max_n, s.Q, s.maxd);
     if (s.kind == 4) return pm1w_smem_bytes(max_n, s.Q, s.maxd);
-    if (s.kind == 6) return pm1q_smem_bytes(max_n, s.Q);
+    if (s.kind == 6) return pm1q_layout(s.block, max_n, s.Q, s.maxd).bytes;
     return sweep_smem_bytes(max_n, s.Q, thr_stride, max_deg, s.stage != 0);
 }
 inline cudaError_t launch_sweep_shape(const SweepLaunch &L, const SweepShape &s, bool pm1, int grid, size_t smem,
@@ -440,16 +462,16 @@ inline cudaError_t launch_sweep_shape(const SweepLaunch &L, const SweepShape &s,
     if (s.kind == 1) return launch_sweep_pm1(L, s.block, s.nslot, s.maxd, s.stage, grid, smem, st);
     if (s.kind == 2) return launch_sweep_pm1s(L, s.block, s.maxd, grid, smem, st);
     if (s.kind == 4) return launch_sweep_pm1w(L, s.Q, s.maxd, s.nslot ? s.nslot : 2, grid, smem, st);
-    if (s.kind == 6) return launch_sweep_pm1q(L, s.block, s.maxd, grid, smem, st);
+    if (s.kind == 6) return launch_sweep_pm1q(L, s.block, s.maxd, s.Q, grid, smem, st);
     return launch_sweep(L, pm1, s.block, grid, smem, st);
 }
-inline int sweep_shape_occupancy(const SweepShape &s, bool pm1, size_t smem)
+inline int sweep_shape_occupancy(const SweepShape &s, bool pm1, int max_n, size_t smem)
 {
     if (s.kind == 5) return sqa_max_active_blocks(s.stage, s.block, s.maxd, s.ncls, s.ent32 != 0, smem);
     if (s.kind == 1) return pm1_max_active_blocks(s.block, s.nslot, s.maxd, s.stage, smem);
     if (s.kind == 2) return pm1s_max_active_blocks(s.block, s.maxd, smem);
     if (s.kind == 4) return pm1w_max_active_blocks(s.Q, s.maxd, s.nslot ? s.nslot : 2, smem);
-    if (s.kind == 6) return pm1q_max_active_blocks(s.block, s.maxd, smem);
+    if (s.kind == 6) return pm1q_max_active_blocks(s.block, s.maxd, max_n, s.Q, smem);
     return sweep_max_active_blocks(pm1, s.block, smem, s.stage != 0);
 }
 
@@ -458,7 +480,7 @@ struct PhaseEngine {
     SweepShape shape;
     size_t sweep_smem;
     bool pm1;
-    int max_n0, max_deg, thr_stride;
+    int max_n0, max_deg, thr_stride, sms;
     const uint32_t *thr;
     const unsigned long long *ent;  // SQA acceptance entries (null for SA)
     int P, W;
@@ -490,8 +512,6 @@ cudaError_t launch_count_single(const DevProb *prob, int n_host, const uint32_t 
 cudaError_t launch_reduce_single(const DevProb *src, DevProb *dst, const int8_t *fixed,
                                  int32_t *old_of_new, int32_t *scratch, cudaStream_t stream);
 int elite_max_samples();
-
-__host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 }  // namespace spvar
 
