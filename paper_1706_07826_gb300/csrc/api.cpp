@@ -619,12 +619,13 @@ int spvar_pticm_sample(const spvar_problem *p, int32_t R, int32_t num_sweeps, co
     if (num_runs == 0) return SPVAR_OK;
     if ((num_sweeps > 0 && !thr) || !final_e || !nkept || !kept_e || (H.n > 0 && (!final_states || !kept)))
         return SPVAR_EINVAL;
-    const size_t smem = pticm_smem_bytes(H.n, R, H.dmax);
-    if (smem > (size_t)device_smem_optin()) return SPVAR_ELIMIT;
+    const size_t optin = (size_t)device_smem_optin();
+    if (pticm_limit_bytes(H.n, R, H.dmax) > optin) return SPVAR_ELIMIT;
+    const size_t smem = pticm_smem_bytes(H.n, R, H.maxdeg, H.dmax);
     cudaStream_t st = as_stream(stream);
     const size_t ntr = 2 * (size_t)(R - keep_from);
     if (ntr > 0) SPVAR_CUDA_TRY(cudaMemsetAsync(nkept, 0, sizeof(int32_t) * ntr * (size_t)num_runs, st));
-    SPVAR_CUDA_TRY(launch_pticm(Pr->dev, thr, thr_stride, xthr, dx, R, num_sweeps, icm_from, keep_from, K, flags, seed,
+    SPVAR_CUDA_TRY(launch_pticm(Pr->dev, H.maxdeg, H.dmax, thr, thr_stride, xthr, dx, R, num_sweeps, icm_from, keep_from, K, flags, seed,
                                 start0, phase, num_runs, smem, kept, kept_e, nkept, final_states, final_e, st));
     return SPVAR_OK;
 }

@@ -67,7 +67,7 @@ cudaError_t engine_phase(const PhaseEngine &E, Slot *slots, int nslots, int T, i
     L.W = E.W;
     if (E.ev_sweep[0] && (e = record(E.ev_sweep[0])) != cudaSuccess) return e;
     // the sampler: persistent sweep launch over the work items, or one PTICM run per start
-    e = E.pt_R > 0 ? launch_pticm_slots(slots, nslots, C.Smax, E.pt_thr, E.thr_stride, E.pt_xthr, E.pt_dx, E.pt_R, T,
+    e = E.pt_R > 0 ? launch_pticm_slots(slots, nslots, C.Smax, E.max_deg, E.pt_dmax, E.pt_thr, E.thr_stride, E.pt_xthr, E.pt_dx, E.pt_R, T,
                                         E.pt_K, E.pt_smem, st)
                    : launch_sweep_shape(L, E.shape, E.pm1, grid, E.sweep_smem, st);
     if (e != cudaSuccess) return e;
@@ -249,6 +249,7 @@ PhaseEngine engine_of(const spvar_plan *pl)
     E.pt_R = pl->pt_R;
     E.pt_K = pl->pt_K;
     E.pt_dx = pl->pt_dx;
+    E.pt_dmax = pl->dmax;
     E.pt_thr = pl->d_pt_thr;
     E.pt_xthr = pl->d_pt_xthr;
     E.pt_smem = pl->pt_smem;
@@ -634,12 +635,11 @@ int spvar_plan_create(const spvar_problem *const *problems, int32_t nproblems,
         pl->pt_K = p.pticm_keep;
         for (const Problem *P : pl->probs) {
             if (P->hdr.n > pticm_max_n() || p.pticm_temps > pticm_max_r()) { delete pl; return SPVAR_ELIMIT; }
-            pl->pt_smem = std::max(pl->pt_smem, pticm_smem_bytes(P->hdr.n, p.pticm_temps, P->hdr.dmax));
             pl->pt_dx = std::max(pl->pt_dx, (int)std::min<long long>((long long)P->hdr.n * P->hdr.dmax, 1 << 30));
         }
-        pl->pt_smem = std::max(pl->pt_smem, pticm_smem_bytes(pl->max_n0, p.pticm_temps, dmax));
         pl->pt_dx = std::max(pl->pt_dx, 1);
-        if (pl->pt_smem > (size_t)optin) { delete pl; return SPVAR_ELIMIT; }
+        if (pticm_limit_bytes(pl->max_n0, p.pticm_temps, dmax) > (size_t)optin) { delete pl; return SPVAR_ELIMIT; }
+        pl->pt_smem = pticm_smem_bytes(pl->max_n0, p.pticm_temps, pl->max_deg, dmax);
     }
     const int nslots = nproblems * p.num_starts;
     SolveConsts &C = pl->C;

@@ -400,13 +400,15 @@ int pm1q_max_active_blocks(int block, int maxd, int max_n, int Q, size_t smem);
 
 // PTICM sampler (sweep_pticm.cu): one CTA per run, every replica's spins in
 // shared memory.
-size_t pticm_smem_bytes(int n, int R, int dmax);
+size_t pticm_limit_bytes(int n, int R, int dmax);
+size_t pticm_smem_bytes(int n, int R, int maxdeg, int dmax);
 // PTICM runs of every start of a slot table (the sampler of Alg. 2 in a plan).
-cudaError_t launch_pticm_slots(Slot *slots, int nslots, int Smax, const uint32_t *thr, int thr_stride,
-                               const uint32_t *xthr, int dx, int R, int T, int K, size_t smem, cudaStream_t st);
+cudaError_t launch_pticm_slots(Slot *slots, int nslots, int Smax, int maxdeg, int dmax, const uint32_t *thr,
+                               int thr_stride, const uint32_t *xthr, int dx, int R, int T, int K, size_t smem,
+                               cudaStream_t st);
 int pticm_max_r();
 int pticm_max_n();
-cudaError_t launch_pticm(const DevProb *prob, const uint32_t *thr, int thr_stride, const uint32_t *xthr, int dx,
+cudaError_t launch_pticm(const DevProb *prob, int maxdeg, int dmax, const uint32_t *thr, int thr_stride, const uint32_t *xthr, int dx,
                          int R, int T, int icm_from, int keep_from, int K, int flags, uint64_t seed,
                          uint32_t start0, uint32_t phase, int runs, size_t smem, uint32_t *kept, int64_t *kept_e,
                          int32_t *nkept, uint32_t *final_bits, int64_t *final_e, cudaStream_t st);
@@ -491,7 +493,7 @@ struct PhaseEngine {
     cudaEvent_t ev_post;  // recorded after each phase's persistence pass (null: none)
     SolveConsts C;
     // PTICM as the sampler (pt_R > 0): one run per start instead of the sweep launch
-    int pt_R = 0, pt_K = 0, pt_dx = 0;
+    int pt_R = 0, pt_K = 0, pt_dx = 0, pt_dmax = 0;
     const uint32_t *pt_thr = nullptr;   // [R][thr_stride]
     const uint32_t *pt_xthr = nullptr;  // [R - 1][pt_dx + 1]
     size_t pt_smem = 0;

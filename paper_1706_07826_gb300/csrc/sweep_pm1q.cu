@@ -37,30 +37,6 @@ constexpr size_t kQuadStatic = 7 << 10;     // static shared memory and the syst
 constexpr size_t kQuadSmemMax = 218 << 10;  // dynamic shared memory records may bring a CTA to (the static part is 6 KB)
 constexpr uint32_t kM = 0x01010101u, kN = 0x11111111u, kOdd = 0x10101010u;
 
-// Shared memory by its 32-bit address: with generic pointers every data-dependent load
-// costs one more instruction, the sum of the 64-bit base and the offset.
-__device__ __forceinline__ uint32_t shared_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t lds(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint2 lds2(uint32_t a)
-{
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint4 lds4(uint32_t a)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(a)
-                 : "memory");
-    return v;
-}
 // NV words (one of every pair of a group) at once.
 template <int NV>
 __device__ __forceinline__ void lds_nv(uint32_t a, uint32_t (&v)[NV])
@@ -77,7 +53,7 @@ template <int NV>
 __device__ __forceinline__ void sts_nv(uint32_t a, const uint32_t (&v)[NV])
 {
     if constexpr (NV == 1) {
-        asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v[0]) : "memory");
+        sts(a, v[0]);
     } else {
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v[0]), "r"(v[1]) : "memory");
     }
