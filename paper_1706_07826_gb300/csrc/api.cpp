@@ -248,6 +248,67 @@ int host_problem_upload(const HostProblem &hp, void *blob, cudaStream_t st, DevP
 
 }  // namespace spvar
 
+namespace {
+
+// Shape of one sample of `quads` quads on a quad-group kernel (pm1: +-1 couplers, else integer
+// ones): block size and quads per item whose busiest SM is done first.  A thread's work per
+// sweep is its rounds of each colour class, a set-up (0.4 of a pair of quads) and the groups
+// of its unit; an SM works its resident warps off four at a time, but a thread's chain of
+// dependent instructions takes as long as four warps a scheduler need (a kernel with fewer
+// is bound by latency).  A lone quad per SM of a large +-1 problem goes to the streaming
+// kernel, whose threads take two spins at once without a set-up.  Measured, 500 sweeps: 3D L =
+// 12 with 250 quads 1.43 ms (1024 threads, pairs) against 1.69 streaming, with 100 quads
+// 1.13 against 0.98 streaming; L = 9 with 50 quads 1.09 against 1.35 streaming.
+SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, bool pm1)
+{
+    const DevProb &H = P->hdr;
+    const int md = H.maxdeg <= 6 ? 6 : 8;
+    SweepShape best{pm1 ? 6 : 7, 0, 1, 0, 0, md};
+    double best_t = 1e300;
+    for (int B : {512, 1024})
+        for (int Q : {1, 2, 4, 8}) {
+            size_t bytes;
+            int per = 1;  // quads of a group
+            double len = 1.0;
+            if (pm1) {
+                const QuadLayout l = pm1q_layout(B, H.n, Q, md);
+                bytes = l.bytes + (7 << 10);
+                per = 2 * l.nv;
+                len = Q == 1 ? 0.55 : l.nv == 2 ? 1.75 : 1.0;
+                if (l.rec == 0) len += 0.7;
+            } else {
+                const GqLayout l = gq_layout(B, H.n, Q, md, thr_stride, (size_t)optin);
+                if (l.nw == 0) continue;
+                bytes = l.bytes + (3 << 10);
+            }
+            if (bytes > (size_t)optin || (Q > 1 && Q % per)) continue;
+            const int groups = ceil_div(Q, per), k = ceil_div(ceil_div(quads, Q), sms);  // items of the busiest SM
+            const int occ = std::min<int>(optin / (int)bytes, 1024 / B), conc = std::min(k, occ);
+            if (occ < 1) continue;
+            double work = 0.0;
+            for (int c = 0; c < H.ncol; ++c) {
+                const double nc = P->csize[c], all = ceil(nc / B) * (0.4 + len * groups);
+                work += std::min(all, ceil(nc * groups / B) * (0.4 + len));
+            }
+            const double t = ceil((double)k / conc) * work * std::max(conc * B / 128.0, 4.0);
+            if (t <= best_t) {
+                best_t = t;
+                best.block = B;
+                best.Q = Q;
+            }
+        }
+    if (pm1 && best.block > 0 && pm1s_shape_ok(512, md, H.n, 1)) {
+        const int bytes = (int)pm1s_smem_bytes(H.n, 1, md) + (2 << 10), k = ceil_div(quads, sms);
+        const int occ = std::min(optin / bytes, 2), conc = std::min(k, occ);
+        double work = 0.0;
+        for (int c = 0; c < H.ncol; ++c) work += 1.86 * ceil(P->csize[c] / 1024.0);
+        if (occ > 0 && ceil((double)k / conc) * work * 4.0 * conc < best_t) best = SweepShape{2, 512, 1, 0, 0, md};
+    }
+    return best;
+}
+
+}  // namespace
+
 extern "C" {
 
 const char *spvar_strerror(int code)
@@ -456,11 +517,8 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
             }
         // large problems: the quad-group kernel, or (large biases) the streaming one (one quad per CTA)
         if (sh.kind == 0 && pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
-            SweepShape c = pm1q_default(H.n, md, (size_t)optin);
-            if (c.block > 0) {
-                c.Q = pm1q_sample_quads(quads, sms, c.Q, pm1q_layout(c.block, H.n, c.Q, md).nv);
-                sh = c;
-            }
+            const SweepShape c = quad_group_shape(P, quads, sms, optin, thr_stride, true);
+            if (c.block > 0) sh = c;
         }
         if (sh.kind == 0 && pm1s_shape_ok(512, md, H.n, 1) &&
             pm1s_smem_bytes(H.n, 1, md) <= (size_t)optin)
@@ -484,6 +542,11 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
             }
         }
     }
+    if (sh.kind == 0 && mode16 == 0 && H.maxdeg <= 8) {
+        // couplers of several magnitudes: the quad-group kernel for integer couplers
+        const SweepShape c = quad_group_shape(P, quads, sms, optin, thr_stride, false);
+        if (c.block > 0) sh = c;
+    }
     if (sh.kind == 0 && sweep_shape_smem(sh, H.n, thr_stride, H.maxdeg) > (size_t)optin) sh.stage = 0;
     const size_t smem = sweep_shape_smem(sh, H.n, thr_stride, H.maxdeg);
     if (smem > (size_t)optin) return SPVAR_ELIMIT;
@@ -502,6 +565,7 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
     L.single.t0 = sweep_begin;
     L.thr = thr;
     L.thr_stride = thr_stride;
+    L.thr_step = thr_stride;
     L.T = num_sweeps;
     L.Q = Q;
     L.stage_ell = sh.stage;

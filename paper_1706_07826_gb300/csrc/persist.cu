@@ -330,13 +330,15 @@ __device__ __forceinline__ int item_quads(const DevProb *P, const SolveConsts &C
                                           long long quads)
 {
     if (C.fit_words > 0) {
-        const int fit = min(64, max(1, 2 * pm1q_fit_pairs(C.fit_words, P->n, C.fit_rec, C.fit_nv)));
-        const int step = 2 * C.fit_nv, per = C.fit_nv == 1 ? 4 : 7;
+        const bool pairs = C.fit_nv > 0;  // else single quads of -fit_nv words a spin
+        const int fit = min(64, max(1, pairs ? 2 * pm1q_fit_pairs(C.fit_words, P->n, C.fit_rec, C.fit_nv)
+                                             : (C.fit_words - C.fit_rec * P->n) / gq_quad_words(P->n, -C.fit_nv)));
+        const int step = pairs ? 2 * C.fit_nv : 1, per = C.fit_nv > 1 ? 7 : pairs ? 4 : 2;
         const float share = (float)load / ((float)max(P->n, 1) * (float)C.sms);  // quads of this size per SM
         int best = 1;
         float best_t = 3e38f;
-        for (int q = C.fit_nv == 1 ? 1 : step; q <= max(fit, step) && q < nquads + step; q += q == 1 ? 1 : step) {
-            const float cost = q == 1 ? 3.f : (float)(per * ceil_div(q, step) + 1);
+        for (int q = C.fit_nv <= 1 ? 1 : step; q <= max(fit, step) && q < nquads + step; q += q == 1 ? 1 : step) {
+            const float cost = q == 1 && pairs ? 3.f : (float)(per * ceil_div(q, step) + 1);
             const float t = quads <= (long long)C.sms * q ? cost : cost * (share / (float)q + 0.5f);
             if (t < best_t) {
                 best_t = t;

@@ -41,6 +41,12 @@ cudaError_t engine_phase(const PhaseEngine &E, Slot *slots, int nslots, int T, i
     C.fit_nslot = E.shape.kind == 1 ? E.shape.nslot : 0;
     QuadLayout ql{1, 0, 0, 0, 0};
     if (E.shape.kind == 6) ql = pm1q_layout(E.shape.block, E.max_n0, E.shape.Q, E.shape.maxd);
+    if (E.shape.kind == 7) {
+        const GqLayout gl = gq_layout(E.shape.block, E.max_n0, E.shape.Q, E.shape.maxd, E.thr_stride, kSmemOptin);
+        ql.fit_words = gl.fit_words;
+        ql.rec = gl.rec;
+        ql.nv = -gl.nw;
+    }
     C.fit_words = ql.fit_words;
     C.fit_rec = ql.rec;
     C.fit_nv = ql.nv;
@@ -57,6 +63,7 @@ cudaError_t engine_phase(const PhaseEngine &E, Slot *slots, int nslots, int T, i
     L.queue = E.ctr + 1;
     L.thr = E.thr;
     L.thr_stride = E.thr_stride;
+    L.thr_step = E.thr_step;
     L.T = T;
     L.Q = E.shape.Q;
     L.stage_ell = E.shape.stage;
@@ -97,6 +104,7 @@ struct spvar_plan {
     std::vector<int> starts_of;  // slot -> problem
     spvar_params prm{};
     SolveConsts C{};
+    int trial_rows = 1;  // rows of the schedule per sweep (more than one in the autotuner's trials)
     int T = 0, thr_stride = 1, max_n0 = 0, max_deg = 1, iters_max = 1;
     int ncol_max = 0, class_max = 0;  // most colour classes and largest class of any problem
     int jabs_max = 0;                 // largest coupler magnitude of any problem
@@ -219,7 +227,7 @@ void solve_cache_put(std::vector<int64_t> key, spvar_plan *pl)
 
 int grid_for(const spvar_plan *pl, int items)
 {
-    const int occ = std::max(1, sweep_shape_occupancy(pl->shape, pl->pm1, pl->max_n0, pl->sweep_smem));
+    const int occ = std::max(1, sweep_shape_occupancy(pl->shape, pl->pm1, pl->max_n0, pl->thr_stride, pl->sweep_smem));
     const int full = occ * pl->sms;
     if (!pl->shape.balance || items <= full) return std::max(1, std::min(items, full));
     return ceil_div(items, ceil_div(items, full));
@@ -235,6 +243,7 @@ PhaseEngine engine_of(const spvar_plan *pl)
     E.max_deg = pl->max_deg;
     E.sms = pl->sms;
     E.thr_stride = pl->thr_stride;
+    E.thr_step = pl->thr_stride * pl->trial_rows;
     E.thr = pl->d_thr;
     E.ent = pl->d_ent;
     E.P = pl->sqa_P;
@@ -397,6 +406,26 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
                 out.push_back(sh);
         }
     }
+    // few quads: the streaming kernel too (3D L = 9, one start of 69 samples, 114 sweeps: 0.67 ms
+    // against 0.94 for the quad-group kernel)
+    if (quads_ok && pl->C.nslots * ceil_div(pl->C.Smax, 4) <= 2 * pl->sms) {
+        const int md = pl->max_deg <= 6 ? 6 : 8;
+        for (int b : {256, 512, 1024}) {
+            SweepShape sh{2, b, 1, 0, 0, md};
+            if (pm1s_shape_ok(b, md, pl->max_n0, 1) &&
+                sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
+                out.push_back(sh);
+        }
+    }
+    // couplers of several magnitudes: the quad-group kernel for integer couplers (Gaussian x 100 on 3D
+    // L = 9, 1000 samples: 2.8 ms against 5.1 for the general kernel)
+    if (!quads_ok && pl->max_deg <= 8) {
+        const int md = pl->max_deg <= 6 ? 6 : 8;
+        const int shapes[][2] = {{256, 1}, {256, 2}, {256, 4}, {512, 1}, {512, 2}, {512, 4}, {512, 8}, {1024, 1}, {1024, 2}, {1024, 8}};
+        for (const auto &bq : shapes)
+            if (gq_layout(bq[0], pl->max_n0, bq[1], md, pl->thr_stride, (size_t)optin).nw > 0)
+                out.push_back(SweepShape{7, bq[0], bq[1], 0, 0, md});
+    }
     const bool others = out.size() == listed;
     if (others && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
         const int md = pl->max_deg <= 6 ? 6 : 8;
@@ -460,7 +489,7 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
     return out;
 }
 
-// Times a short run of the plan's phases (at most 4, at most 64 sweeps each;
+// Times a short run of the plan's phases (at most 4, at most 512 sweeps each;
 // the best of two repetitions after an untimed one, and one discarded trial
 // before the first candidate) for every candidate shape and keeps the fastest;
 // results are cached per problem/plan geometry.
@@ -479,7 +508,15 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
             return;
         }
     }
-    const int Tt = std::min(pl->T, 64);
+    int Tt = std::min(pl->T, 128);
+    // the trials run through the whole schedule in Tt sweeps, so that their reductions leave about as many
+    // spins as the run's: on its first Tt rows (high temperatures) hardly a spin is fixed, and shapes that
+    // suit the full problem but not the small one of the solving phase won by up to 26 %
+    auto set_sweeps = [&](int t) {
+        Tt = std::min(pl->T, t);
+        pl->trial_rows = std::max(1, pl->T / std::max(Tt, 1));
+    };
+    set_sweeps(128);
     float best = 1e30f;
     SweepShape pick{0, 256, 1, 0, 0, 0};
     bool found = false;
@@ -498,7 +535,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
     auto trial = [&](const SweepShape &sh, int chunk_t) -> float {
         pl->shape = sh;
         pl->sweep_smem = sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg);
-        if (sweep_shape_occupancy(sh, pl->pm1, pl->max_n0, pl->sweep_smem) < 1) return 1e30f;
+        if (sweep_shape_occupancy(sh, pl->pm1, pl->max_n0, pl->thr_stride, pl->sweep_smem) < 1) return 1e30f;
         const int nslots = (pl->prm.form == SPVAR_FORM_PLAIN) ? 1 : pl->C.nslots;
         pl->C.Q = sh.Q;
         pl->C.chunk = chunk_t;
@@ -525,12 +562,25 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
         return ms;
     };
     // one discarded trial first: clocks and caches settle before the timed candidates
-    if (!cands.empty()) trial(cands.front(), 0);
-    for (const SweepShape &sh : cands) {
-        const float ms = trial(sh, 0);
+    // (and, where a trial is short, it says how many more sweeps make it a millisecond: below that launches and
+    // their gaps, which a run's graph does not have, decide between nearly equal shapes)
+    if (!cands.empty()) {
+        const float ms = trial(cands.front(), 0);
+        if (ms < 1.0f) set_sweeps(128 * std::min(4, (int)(1.0f / std::max(ms, 0.1f)) + 1));
+    }
+    std::vector<std::pair<float, size_t>> times;
+    for (size_t i = 0; i < cands.size(); ++i) {
+        const float ms = trial(cands[i], 0);
+        if (ms < 1e30f) times.emplace_back(ms, i);
+    }
+    // the candidates within 5 % of the best, at most four, once more: single trials of nearly
+    // equal shapes pick one that is up to 4 % slower
+    std::sort(times.begin(), times.end());
+    for (size_t k = 0; k < times.size() && k < 4 && times[k].first <= 1.05f * times[0].first; ++k) {
+        const float ms = std::min(times[k].first, trial(cands[times[k].second], 0));
         if (ms < best) {
             best = ms;
-            pick = sh;
+            pick = cands[times[k].second];
             found = true;
         }
     }
@@ -540,6 +590,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
         const float ms4 = trial(pick, ceil_div(Tt, 4));
         if (ms4 < best) pick.lpp = 4;
     }
+    pl->trial_rows = 1;
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     if (!found) pick = SweepShape{0, 256, 1, 0, 0, 0};
@@ -1045,8 +1096,13 @@ int spvar_plan_shape(const spvar_plan *plan, int32_t *block, int32_t *replicas_p
     if (replicas_per_block) *replicas_per_block = 4 * plan->shape.Q;
     if (staged) {
         const int k = plan->shape.kind;
-        *staged = k == 1 ? 2 : k == 2 ? 3 : k == 4 ? 4 : k == 5 ? (plan->shape.stage >= 2 ? 6 : 5) : k == 6 ? 7
-                                                                                                 : plan->shape.stage;
+        *staged = k == 1   ? 2
+                  : k == 2 ? 3
+                  : k == 4 ? 4
+                  : k == 5 ? (plan->shape.stage >= 2 ? 6 : 5)
+                  : k == 6 ? 7
+                  : k == 7 ? 8
+                           : plan->shape.stage;
     }
     if (grid) *grid = plan->sweep_grid;
     return SPVAR_OK;

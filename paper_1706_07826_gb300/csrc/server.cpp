@@ -529,6 +529,15 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
         Q = E.shape.Q;
         chosen = true;
     }
+    // any couplers: the quad-group kernel for integer couplers where it applies
+    const bool auto_gq = !pm1_only && p.sweep_kernel == SPVAR_SWEEP_AUTO && p.sweep_block == 0 &&
+                         p.replicas_per_block == 0 && cfg->max_degree <= 8 &&
+                         gq_default(cfg->max_n, md, stride, (size_t)optin).block > 0;
+    if (auto_gq) {
+        E.shape = gq_default(cfg->max_n, md, stride, (size_t)optin);
+        Q = E.shape.Q;
+        chosen = true;
+    }
     if (!chosen && pm1_only && cfg->max_degree <= 8 && cfg->max_dmax <= 254 && pm1s_shape_ok(blk, md, cfg->max_n, 1)) {
         SweepShape sh{2, blk, 1, 0, 0, md};
         if (sweep_shape_smem(sh, cfg->max_n, stride, cfg->max_degree) <= (size_t)optin) {
@@ -562,6 +571,7 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
     E.max_deg = cfg->max_degree;
     E.sms = S->sms;
     E.thr_stride = stride;
+    E.thr_step = stride;
     E.thr = (const uint32_t *)(w + o_thr);
     E.jobs = (SweepJob *)(w + o_jobs);
     E.items = (WorkItem *)(w + o_items);
@@ -586,12 +596,12 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
         t.E = E;
         t.E.max_n0 = tn;
         t.E.C.max_n0 = tn;
-        if (auto_quads && !sqa) {
-            t.E.shape = pm1q_default(tn, md, (size_t)optin);
+        if ((auto_quads || auto_gq) && !sqa) {
+            t.E.shape = auto_gq ? gq_default(tn, md, stride, (size_t)optin) : pm1q_default(tn, md, (size_t)optin);
             t.E.C.Q = t.E.shape.Q;
         }
         t.E.sweep_smem = sweep_shape_smem(t.E.shape, tn, stride, cfg->max_degree);
-        const int occ = std::max(1, sweep_shape_occupancy(t.E.shape, t.E.pm1, tn, t.E.sweep_smem));
+        const int occ = std::max(1, sweep_shape_occupancy(t.E.shape, t.E.pm1, tn, stride, t.E.sweep_smem));
         t.grid = occ * S->sms;
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(S->cap_st, cudaStreamCaptureModeRelaxed) == cudaSuccess) {

@@ -16,6 +16,7 @@ namespace spvar {
 constexpr int kMaxColours = SPVAR_MAX_DEGREE + 1;
 constexpr uint32_t kSweepBits = 20;                 // counter word 1 = phase << 20 | sweep
 constexpr uint32_t kInitSlot = (1u << kSweepBits) - 1u;
+constexpr size_t kSmemOptin = 227 << 10;            // shared memory of one CTA
 
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
@@ -98,7 +99,8 @@ struct SweepLaunch {
     int32_t *queue;         // device atomic cursor (queue mode)
     SweepJob single;
     const uint32_t *thr;
-    int32_t thr_stride, T, Q, stage_ell;
+    int32_t thr_stride, T, Q, stage_ell;  // thr_stride: entries of a row
+    int32_t thr_step;       // words from one sweep's row to the next
     int32_t max_n;          // largest n of any job (shared-memory carve-up)
     int32_t max_deg;        // largest maxdeg of any job (staged ELL size)
     // simulated quantum annealing: acceptance entries [T][3][W], Trotter slices, chosen slice per sample
@@ -157,7 +159,7 @@ struct SolveConsts {
     // threads x nslot items per thread, colour classes in whole slots); 0: Q quads
     int32_t fit_block, fit_nslot, grid;  // grid: CTAs of the sweep launch
     // quad-group kernel: words of the launch's shared memory for records and groups (0: another kernel), words
-    // of a spin's record, pairs of quads per group, SMs
+    // of a spin's record, pairs of quads per group (integer-coupler form: minus the words per spin and quad), SMs
     int32_t fit_words, fit_rec, fit_nv, sms;
     // sweeps per phase, and sweeps per launch (0: the whole phase in one launch).  With
     // chunk > 0 a phase's sample is annealed over ceil(T / chunk) launches, each resuming
@@ -360,7 +362,8 @@ inline int sqa_reg_ncls(int ncol, int max_class, int block, int P)
 // (maxd neighbour offsets per spin staged in shared memory, Q = 1), kind 4 =
 // warp-per-quad +-1 kernel (Q = warps = block / 32; nslot = spins in flight per lane,
 // 2 or 4), kind 5 = simulated
-// quantum annealing (Q = 1).  A persistent grid holds
+// quantum annealing (Q = 1), kind 6 = quad-group +-1 kernel, kind 7 = quad-group kernel
+// for integer couplers (Q = quads of the largest problem per item).  A persistent grid holds
 // every CTA the SMs can keep resident, or (balance) the fewest CTAs that still
 // need the same number of waves of items, so that no last wave runs nearly empty.
 struct SweepShape {
@@ -392,11 +395,23 @@ struct QuadLayout {
 };
 QuadLayout pm1q_layout(int block, int max_n, int Q, int maxd);
 SweepShape pm1q_default(int max_n, int maxd, size_t optin);
-int pm1q_sample_quads(int quads, int sms, int Q, int nv);
 // A requested item of Q quads is taken where two copies of every quad's spin words fit a CTA.
 inline bool pm1q_request_ok(int max_n, int Q, size_t optin) { return 8 * (size_t)Q * ((size_t)max_n + 1) <= optin; }
 cudaError_t launch_sweep_pm1q(const SweepLaunch &L, int block, int maxd, int Q, int grid, size_t smem, cudaStream_t st);
 int pm1q_max_active_blocks(int block, int maxd, int max_n, int Q, size_t smem);
+
+// Quad-group sweep for integer couplers (sweep_gq.cu): degree <= 8, dmax <= 16382, up to
+// 64 quads of one problem per work item.
+__host__ __device__ inline int gq_quad_words(int n, int nw) { return (8 + nw * n + 3) & ~3; }
+struct GqLayout {
+    int nw, rec, unit_rows;  // words per spin and quad (0: the kernel does not apply), of a record, listed rounds of units
+    int fit_words;           // words for records and quads
+    size_t bytes;            // dynamic shared memory
+};
+GqLayout gq_layout(int block, int max_n, int Q, int maxd, int thr_stride, size_t optin);
+SweepShape gq_default(int max_n, int maxd, int thr_stride, size_t optin);
+cudaError_t launch_sweep_gq(const SweepLaunch &L, int block, int maxd, int Q, int grid, size_t smem, cudaStream_t st);
+int gq_max_active_blocks(int block, int maxd, int thr_stride, size_t smem);
 
 // PTICM sampler (sweep_pticm.cu): one CTA per run, every replica's spins in
 // shared memory.
@@ -455,6 +470,7 @@ inline size_t sweep_shape_smem(const SweepShape &s, int max_n, int thr_stride, i
     if (s.kind == 2) return pm1s_smem_bytes(max_n, s.Q, s.maxd);
     if (s.kind == 4) return pm1w_smem_bytes(max_n, s.Q, s.maxd);
     if (s.kind == 6) return pm1q_layout(s.block, max_n, s.Q, s.maxd).bytes;
+    if (s.kind == 7) return gq_layout(s.block, max_n, s.Q, s.maxd, thr_stride, kSmemOptin).bytes;
     return sweep_smem_bytes(max_n, s.Q, thr_stride, max_deg, s.stage != 0);
 }
 inline cudaError_t launch_sweep_shape(const SweepLaunch &L, const SweepShape &s, bool pm1, int grid, size_t smem,
@@ -465,15 +481,17 @@ inline cudaError_t launch_sweep_shape(const SweepLaunch &L, const SweepShape &s,
     if (s.kind == 2) return launch_sweep_pm1s(L, s.block, s.maxd, grid, smem, st);
     if (s.kind == 4) return launch_sweep_pm1w(L, s.Q, s.maxd, s.nslot ? s.nslot : 2, grid, smem, st);
     if (s.kind == 6) return launch_sweep_pm1q(L, s.block, s.maxd, s.Q, grid, smem, st);
+    if (s.kind == 7) return launch_sweep_gq(L, s.block, s.maxd, s.Q, grid, smem, st);
     return launch_sweep(L, pm1, s.block, grid, smem, st);
 }
-inline int sweep_shape_occupancy(const SweepShape &s, bool pm1, int max_n, size_t smem)
+inline int sweep_shape_occupancy(const SweepShape &s, bool pm1, int max_n, int thr_stride, size_t smem)
 {
     if (s.kind == 5) return sqa_max_active_blocks(s.stage, s.block, s.maxd, s.ncls, s.ent32 != 0, smem);
     if (s.kind == 1) return pm1_max_active_blocks(s.block, s.nslot, s.maxd, s.stage, smem);
     if (s.kind == 2) return pm1s_max_active_blocks(s.block, s.maxd, smem);
     if (s.kind == 4) return pm1w_max_active_blocks(s.Q, s.maxd, s.nslot ? s.nslot : 2, smem);
     if (s.kind == 6) return pm1q_max_active_blocks(s.block, s.maxd, max_n, s.Q, smem);
+    if (s.kind == 7) return gq_max_active_blocks(s.block, s.maxd, thr_stride, smem);
     return sweep_max_active_blocks(pm1, s.block, smem, s.stage != 0);
 }
 
@@ -483,6 +501,7 @@ struct PhaseEngine {
     size_t sweep_smem;
     bool pm1;
     int max_n0, max_deg, thr_stride, sms;
+    int thr_step;  // words from one sweep's acceptance row to the next (thr_stride but in the autotuner's trials)
     const uint32_t *thr;
     const unsigned long long *ent;  // SQA acceptance entries (null for SA)
     int P, W;

@@ -141,7 +141,7 @@ __device__ void run_item(const SweepLaunch &L, const SweepJob &job, int quad0, i
     init_spins(P, job, quad0, nq, sw, nullptr);
     const int t0 = job.t0;
     if (t0 < T)
-        for (int d = tid; d < thr_w; d += B) thr_s[(t0 & 1) * L.thr_stride + d] = L.thr[(size_t)t0 * L.thr_stride + d];
+        for (int d = tid; d < thr_w; d += B) thr_s[(t0 & 1) * L.thr_stride + d] = L.thr[(size_t)t0 * L.thr_step + d];
     __syncthreads();
 
     for (int t = t0; t < T; ++t) {
@@ -150,7 +150,7 @@ __device__ void run_item(const SweepLaunch &L, const SweepJob &job, int quad0, i
         for (int c = 0; c < ncol; ++c) {
             if (c == 0 && t + 1 < T) {
                 uint32_t *nxt = thr_s + ((t + 1) & 1) * L.thr_stride;
-                const uint32_t *src = L.thr + (size_t)(t + 1) * L.thr_stride;
+                const uint32_t *src = L.thr + (size_t)(t + 1) * L.thr_step;
                 for (int d = tid; d < thr_w; d += B) nxt[d] = src[d];
             }
             const int lo = s_cptr[c];

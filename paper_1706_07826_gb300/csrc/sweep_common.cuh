@@ -36,6 +36,10 @@ __device__ __forceinline__ void sts(uint32_t a, uint32_t v)
 {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
+__device__ __forceinline__ void sts2(uint32_t a, uint2 v)
+{
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
 
 // Twice the energy contribution of one spin for the four replicas of a word:
 // s_i (h_i + f_i) with f_i = h_i + sum_j J_ij s_j  (summed over i this is 2E).

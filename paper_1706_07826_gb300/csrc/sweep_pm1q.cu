@@ -25,7 +25,7 @@
 // 2000 + 2000 samples, 1000 sweeps: 271 ms with one quad per word and no records,
 // 174 ms now (1.2e12 attempts/s).
 // Eligible when every |J| = 1, degree <= MAXD <= 8 and dmax <= 30.
-#include "sweep_common.cuh"
+#include "quad_units.cuh"
 
 namespace spvar {
 
@@ -55,7 +55,7 @@ __device__ __forceinline__ void sts_nv(uint32_t a, const uint32_t (&v)[NV])
     if constexpr (NV == 1) {
         sts(a, v[0]);
     } else {
-        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v[0]), "r"(v[1]) : "memory");
+        sts2(a, make_uint2(v[0], v[1]));
     }
 }
 
@@ -80,35 +80,8 @@ struct QuadSmem {
     int zero[2];                 // the row holds a threshold of 0
     int c8lo, c8hi;              // range of the problem's flip-cost constants
     int e2[4 * kQcap];
-    int4 cls[kMaxColours];  // per colour class: first position, spins, rounds of the block, first unit row (-1: none)
+    int4 cls[kMaxColours];  // per colour class, as unit_classes fills it
 };
-
-// How a colour class of nc spins is dealt over the block for np pairs of quads.
-// Units (spin, group g of pairs g, g + G, ...) fill full rounds of B threads; the
-// units left for a last partial round are each split into G2 sub-units (every
-// G2-th pair of the unit's group), so that round uses the whole block.  G is the
-// choice, within `most` rounds, that minimises the rounds' length, a unit's set-up
-// counted as a fifth of a pair.  Returns (G, full units, remainder units, G2).
-__device__ __forceinline__ int4 class_split(int nc, int np, int B, int most)
-{
-    int best = 0x7FFFFFFF;
-    int4 pick = make_int4(1, 0, 0, 1);
-    for (int G = 1; G <= np; ++G) {
-        const int ppu = (np + G - 1) / G;
-        const int U = nc * G, R = U / B, Ur = U - R * B;
-        if (G > 1 && R + (Ur > 0) > most) break;
-        int cost = R * (5 * ppu + 1), G2 = 1;
-        if (Ur > 0) {
-            G2 = max(1, min(ppu, B / Ur));
-            cost += 5 * ((ppu + G2 - 1) / G2) + 1;
-        }
-        if (cost < best) {
-            best = cost;
-            pick = make_int4(G, R * B, Ur, G2);
-        }
-    }
-    return pick;
-}
 
 // One quad's four acceptance tests: adds 1 << (8r + SH) to rej for every replica r whose
 // word is not below its threshold.
@@ -398,7 +371,7 @@ __device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int qua
     const uint32_t phase_hi = job.phase << kSweepBits;
     const uint32_t k0w = k0 + kPhiloxW0, k1w = k1 + kPhiloxW1;
     const uint32_t *__restrict__ thr = L.thr;
-    const size_t ts = (size_t)L.thr_stride;
+    const size_t ts = (size_t)L.thr_step;
     // staged: the units of every thread ([unit_rows][B]: position, first group, group step) and the spins'
     // records ([n] uint4, and [n] words for neighbours 6 and 7); then the pairs
     uint32_t *unit = smem;
@@ -425,23 +398,7 @@ __device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int qua
             sm.zero[t0 & 1] = 0;
         }
     }
-    if (tid == B - 1) {
-        // a class's units are listed while its rounds fit its share of the list; longer classes are
-        // walked a spin per thread, every pair at once
-        int row = 0;
-        for (int c = 0; c < ncol; ++c) {
-            const int lo = P->cptr[c], nc = P->cptr[c + 1] - lo, plain = (nc + B - 1) / B;
-            int4 k = make_int4(lo, nc, plain, -1);
-            const int most = (unit_rows - row) / (ncol - c);
-            if (STAGED && plain <= most && ng > 1) {
-                const int4 sp = class_split(nc, ng, B, most);
-                k.z = (sp.y + sp.z * sp.w + B - 1) / B;
-                k.w = row;
-                row += k.z;
-            }
-            sm.cls[c] = k;
-        }
-    }
+    if (tid == B - 1) unit_classes<B>(P, ncol, ng, unit_rows, sm.cls);
     if (STAGED)
         for (int p = tid; p < n; p += B) {
             const uint32_t meta = g_meta[p];
@@ -498,26 +455,7 @@ __device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int qua
             for (int i = tid; i < 16 * (sm.c8hi - sm.c8lo + 1); i += B)
                 sm.tab[t0 & 1][tab_word(sm.c8lo + (i >> 4), i & 15)] = top_word(row, sm.c8lo + (i >> 4), i & 15, bias);
     }
-    if (STAGED)
-        for (int c = 0; c < ncol; ++c) {
-            const int4 k = sm.cls[c];
-            if (k.w < 0) continue;
-            const int4 sp = class_split(k.y, ng, B, (unit_rows - k.w) / (ncol - c));
-            for (int r = 0; r < k.z; ++r) {
-                const int u = r * B + tid;
-                uint32_t d = 0xFF0000u;  // no unit: the first pair is past the last
-                if (u < sp.y + sp.z * sp.w) {
-                    int uu = u, j = 0;
-                    if (u >= sp.y) {
-                        j = (u - sp.y) / sp.z;
-                        uu = u - j * sp.z;
-                    }
-                    const int g = uu / k.y, step = u < sp.y ? sp.x : sp.x * sp.w;
-                    d = (uint32_t)(k.x + uu - g * k.y) | (uint32_t)(g + j * sp.x) << 16 | (uint32_t)step << 24;
-                }
-                unit[(k.w + r) * B + tid] = d;
-            }
-        }
+    if (STAGED) unit_list<B>(ncol, ng, unit_rows, sm.cls, unit);
     __syncthreads();
 
     QuadItem I;
@@ -634,22 +572,6 @@ SweepShape pm1q_default(int max_n, int maxd, size_t optin)
     for (int Q : {2, 1})
         if (pm1q_layout(1024, max_n, Q, maxd).bytes + kQuadStatic <= optin) return SweepShape{6, 1024, Q, 0, 0, maxd};
     return SweepShape{6, 0, 1, 0, 0, maxd};
-}
-
-// Quads per item of one sample of `quads` quads: the largest share Q finishes first where
-// it needs no more rounds of the SMs for its length (an item's length as in the work list).
-int pm1q_sample_quads(int quads, int sms, int Q, int nv)
-{
-    const int step = 2 * nv, per = nv == 1 ? 4 : 7;
-    int best = step, best_t = 0x7FFFFFFF;
-    for (int q = nv == 1 ? 1 : step; q <= std::max(Q, step); q += q == 1 ? 1 : step) {
-        const int t = (q == 1 ? 3 : per * ceil_div(q, step) + 1) * ceil_div(ceil_div(quads, q), sms);
-        if (t <= best_t) {
-            best_t = t;
-            best = q;
-        }
-    }
-    return std::min(best, Q);
 }
 
 cudaError_t launch_sweep_pm1q(const SweepLaunch &L, int block, int maxd, int Q, int grid, size_t smem, cudaStream_t st)

@@ -97,7 +97,7 @@ __device__ void run_item_pm1s(const SweepLaunch &L, const SweepJob &job, int qua
     const int t0 = job.t0;
     if (t0 < T)
         for (int e = tid + 1; e <= bias; e += B)
-            trow[(t0 & 1) * kRowWordsS + bias + e] = L.thr[(size_t)t0 * L.thr_stride + 2 * e];
+            trow[(t0 & 1) * kRowWordsS + bias + e] = L.thr[(size_t)t0 * L.thr_step + 2 * e];
     __syncthreads();
 
     const Keys10 K = philox_keys<0>((uint32_t)job.seed, (uint32_t)(job.seed >> 32));
@@ -114,7 +114,7 @@ __device__ void run_item_pm1s(const SweepLaunch &L, const SweepJob &job, int qua
         for (int c = 0; c < ncol; ++c) {
             if (c == 0 && t + 1 < T) {
                 uint32_t *nxt = trow + ((t + 1) & 1) * kRowWordsS;
-                const uint32_t *src = L.thr + (size_t)(t + 1) * L.thr_stride;
+                const uint32_t *src = L.thr + (size_t)(t + 1) * L.thr_step;
                 for (int e = tid + 1; e <= bias; e += B) nxt[bias + e] = src[2 * e];
             }
             const int lo = s_cptr[c];

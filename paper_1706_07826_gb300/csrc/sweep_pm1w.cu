@@ -133,7 +133,7 @@ __device__ void run_item_pm1w(const SweepLaunch &L, const SweepJob &job, int qua
         const int t0 = job.t0;
         if (t0 < T)
             for (int e = lane + 1; e <= bias; e += 32)
-                myrows[(t0 & 1) * kRowW + e - 1] = L.thr[(size_t)t0 * L.thr_stride + 2 * e];
+                myrows[(t0 & 1) * kRowW + e - 1] = L.thr[(size_t)t0 * L.thr_step + 2 * e];
         __syncwarp();
 
         for (int t = t0; t < T; ++t) {
@@ -146,7 +146,7 @@ __device__ void run_item_pm1w(const SweepLaunch &L, const SweepJob &job, int qua
             for (int c = 0; c < ncol; ++c) {
                 if (c == 0 && t + 1 < T) {
                     uint32_t *nxt = myrows + ((t + 1) & 1) * kRowW;
-                    const uint32_t *src = L.thr + (size_t)(t + 1) * L.thr_stride;
+                    const uint32_t *src = L.thr + (size_t)(t + 1) * L.thr_step;
                     for (int e = lane + 1; e <= bias; e += 32) nxt[e - 1] = src[2 * e];
                 }
                 const int lo = s_cptr[c], hi = s_cptr[c + 1];

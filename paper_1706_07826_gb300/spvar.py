@@ -535,7 +535,7 @@ class Plan:
         spl = i32(0)
         _check(lib().spvar_plan_sweeps_per_launch(self.handle, ctypes.byref(spl)), "spvar_plan_sweeps_per_launch")
         return dict(block=b.value, replicas_per_block=r.value, kernel=("general", "general-staged", "pm1-register", "pm1-streaming", "pm1-warp",
-                                                                 "sqa", "sqa-register", "pm1-quads")[s.value],
+                                                                 "sqa", "sqa-register", "pm1-quads", "integer-quads")[s.value],
                     grid=g.value, sweeps_per_launch=spl.value)
 
     def close(self):
