@@ -366,6 +366,7 @@ SweepShape sqa_shape(const spvar_plan *pl, int block, int optin, int variant)
                                                        : pl->pm1);
     const bool ok = kind_ok && (variant < 2 || sh.ncls > 0) &&
                     sqa_shape_ok(variant, block, pl->max_n0, pl->max_deg, pl->sqa_P, pl->sqa_W, sh.ncls) &&
+                    sqa_smem_bytes(pl->max_n0, pl->sqa_P, pl->max_deg, pl->sqa_W, variant ? 1 : 0) <= (size_t)optin &&
                     sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin;
     if (!ok) sh.kind = -1;
     return sh;
@@ -516,7 +517,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
         Tt = std::min(pl->T, t);
         pl->trial_rows = std::max(1, pl->T / std::max(Tt, 1));
     };
-    set_sweeps(128);
+    set_sweeps(pl->sqa_P > 0 ? 64 : 128);
     float best = 1e30f;
     SweepShape pick{0, 256, 1, 0, 0, 0};
     bool found = false;
@@ -566,7 +567,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
     // their gaps, which a run's graph does not have, decide between nearly equal shapes)
     if (!cands.empty()) {
         const float ms = trial(cands.front(), 0);
-        if (ms < 1.0f) set_sweeps(128 * std::min(4, (int)(1.0f / std::max(ms, 0.1f)) + 1));
+        if (ms < 1.0f && pl->sqa_P == 0) set_sweeps(128 * std::min(4, (int)(1.0f / std::max(ms, 0.1f)) + 1));
     }
     std::vector<std::pair<float, size_t>> times;
     for (size_t i = 0; i < cands.size(); ++i) {

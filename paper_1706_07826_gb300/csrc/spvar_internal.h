@@ -337,10 +337,11 @@ int pm1_max_active_blocks(int block, int nslot, int maxd, int mode, size_t smem)
 // couplers (|J| <= 15, dmax <= 254) in register form.
 constexpr int kSqaMaxSlices = 1024;
 bool sqa_shape_ok(int variant, int block, int max_n, int max_deg, int P, int W, int ncls = 0);
-size_t sqa_smem_bytes(int max_n, int P, int maxdeg, int W, bool pm1);
+// (A register form is refused where the walk's shared memory, variant 1, does not fit, though it needs less.)
+size_t sqa_smem_bytes(int max_n, int P, int maxdeg, int W, int variant);
 cudaError_t launch_sweep_sqa(const SweepLaunch &L, int variant, int block, int ncls, bool ent32, int grid,
                              size_t smem, cudaStream_t st);
-int sqa_max_active_blocks(int variant, int block, int max_deg, int ncls, bool ent32, size_t smem);
+int sqa_max_active_blocks(int variant, int block, int max_deg, int ncls, int W, bool ent32, size_t smem);
 // The register form holds one spin of every colour class per thread: two or
 // more slices, at most 4 classes, none larger than the block.  Colour-class
 // slots it needs (2 or 4), 0 if it does not apply.
@@ -465,7 +466,7 @@ inline int pm1_nslot(const Problem *P, int Q, int block)
 }
 inline size_t sweep_shape_smem(const SweepShape &s, int max_n, int thr_stride, int max_deg)
 {
-    if (s.kind == 5) return sqa_smem_bytes(max_n, s.slices, max_deg, s.nslot, s.stage != 0);
+    if (s.kind == 5) return sqa_smem_bytes(max_n, s.slices, max_deg, s.nslot, s.stage);
     if (s.kind == 1) return pm1_smem_bytes(s.stage != 0, thr_stride);
     if (s.kind == 2) return pm1s_smem_bytes(max_n, s.Q, s.maxd);
     if (s.kind == 4) return pm1w_smem_bytes(max_n, s.Q, s.maxd);
@@ -486,7 +487,7 @@ inline cudaError_t launch_sweep_shape(const SweepLaunch &L, const SweepShape &s,
 }
 inline int sweep_shape_occupancy(const SweepShape &s, bool pm1, int max_n, int thr_stride, size_t smem)
 {
-    if (s.kind == 5) return sqa_max_active_blocks(s.stage, s.block, s.maxd, s.ncls, s.ent32 != 0, smem);
+    if (s.kind == 5) return sqa_max_active_blocks(s.stage, s.block, s.maxd, s.ncls, s.nslot, s.ent32 != 0, smem);
     if (s.kind == 1) return pm1_max_active_blocks(s.block, s.nslot, s.maxd, s.stage, smem);
     if (s.kind == 2) return pm1s_max_active_blocks(s.block, s.maxd, smem);
     if (s.kind == 4) return pm1w_max_active_blocks(s.Q, s.maxd, s.nslot ? s.nslot : 2, smem);

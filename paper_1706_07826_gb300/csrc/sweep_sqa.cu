@@ -26,16 +26,20 @@ namespace spvar {
 
 namespace {
 
+// Words of the two acceptance rows (register form: at least two rows of 256 bytes).
+__host__ __device__ inline size_t sqa_row_words(int W, bool reg) { return reg && 12 * W < 128 ? 128 : 12 * (size_t)W; }
+
 // Shared memory of one CTA, in 32-bit words: the two 64-bit acceptance rows
 // (current and next sweep), spin words [P][n + 1] (word n of every slice is
 // zero: the target of missing neighbours), for +-1 couplers their inverted
 // copy [P][n + 1], per-spin meta and index, 16-bit neighbour offsets, per-slice
 // energy sums and the chosen slices.
-__host__ __device__ inline size_t sqa_words(int max_n, int P, int maxdeg, int W, bool pm1)
+__host__ __device__ inline size_t sqa_words(int max_n, int P, int maxdeg, int W, bool pm1, bool reg)
 {
     const size_t slice = (size_t)max_n + 1;
-    size_t w = 2 * 2 * 3 * (size_t)W;  // two rows of 3W 64-bit entries
+    size_t w = sqa_row_words(W, reg);
     w += (size_t)P * slice * (pm1 ? 2 : 1);
+    if (reg) return w + 4 * (size_t)P + 4;
     w += 2 * (size_t)max_n;
     if (pm1) w += ((size_t)(maxdeg <= 6 ? 6 : 8) * max_n + 1) / 2;  // the kernel's unrolled degree
     return w + 4 * (size_t)P + 4;
@@ -61,15 +65,6 @@ __device__ __forceinline__ uint32_t madq(uint32_t a, uint32_t b, uint32_t c)
     asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
-__device__ __forceinline__ uint32_t lds_q(const uint32_t *base, uint32_t byte_off)
-{
-    return *reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(base) + byte_off);
-}
-__device__ __forceinline__ void sts_q(uint32_t *base, uint32_t byte_off, uint32_t v)
-{
-    *reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(base) + byte_off) = v;
-}
-
 // Register-resident form, +-1 couplers: the thread's spin of one colour class
 // (its word offsets, flip-cost constant and spin word of the counter held in
 // registers) in slices PAR + 2 (g + G m), m = 0, 1, ...  Byte offsets:
@@ -85,13 +80,16 @@ struct SqaRegConsts {
 // and the acceptance of all of them, then the stores.  `chain`: the items are
 // consecutive slices of the thread's sequence (tau, tau + 2, ...), so the
 // down neighbour of one is the up neighbour of the one before (`prev_up`,
-// valid when `have`).  E32: acceptance entries are 32-bit (no entry of the
-// table is 2^32, i.e. every flip has a nonzero acceptance probability).
+// valid when `have`).  E: form of the acceptance rows.  0: 64-bit entries as in the table.
+// Where no entry of the table is 2^32 (every flip has a nonzero acceptance
+// probability) the row holds 2^32 - 1 - entry, the largest word accepted, in 32 bits and
+// one comparison accepts: E = 1 by entry index, E = 2 (3W <= 64 entries) with the index formed
+// as a byte offset that the byte permute merges with the address of the 256-byte row.
 // SI: small integer couplers (|J| <= 15; jp holds |J| of neighbour d in bits
 // 4d .. 4d + 3): the byte-wise neighbour sum is weighted, X = sum |J| b', and
 // the entry index a W + k is formed per replica (it may exceed a byte).
-template <int PAR, int MAXD, int U, bool E32, bool SI>
-__device__ __forceinline__ void sqa_reg_items(uint32_t *sw, const void *entv, int P, const int (&tau)[U],
+template <int PAR, int MAXD, int U, int E, bool SI>
+__device__ __forceinline__ void sqa_reg_items(uint32_t row, int P, const int (&tau)[U],
                                               const uint32_t (&base)[U], const uint32_t (&iw)[U], uint32_t own4,
                                               const uint32_t (&o4)[MAXD], uint32_t c0, uint32_t jp,
                                               const SqaRegConsts &K, const PhiloxKeys<2> &Kr, bool chain, bool have, uint32_t &prev_up)
@@ -101,7 +99,7 @@ __device__ __forceinline__ void sqa_reg_items(uint32_t *sw, const void *entv, in
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         oa[u] = base[u] + own4;
-        own[u] = lds_q(sw, oa[u]);
+        own[u] = lds(oa[u]);
         // slice neighbours; only the first even slice (down) and the last odd one (up) wrap
         uint32_t ua = oa[u] + K.ns4, da = oa[u] - K.ns4;
         if (PAR == 0) {
@@ -109,13 +107,13 @@ __device__ __forceinline__ void sqa_reg_items(uint32_t *sw, const void *entv, in
         } else {
             if (tau[u] == P - 1) ua = oa[u] - K.wrap4;
         }
-        up[u] = lds_q(sw, ua);
+        up[u] = lds(ua);
         if (chain && (u > 0 || have)) dn[u] = u > 0 ? up[u - 1] : prev_up;
-        else dn[u] = lds_q(sw, da);
+        else dn[u] = lds(da);
         x[u] = 0;
 #pragma unroll
         for (int d = 0; d < MAXD; ++d) {
-            const uint32_t w = lds_q(sw, base[u] + o4[d]);
+            const uint32_t w = lds(base[u] + o4[d]);
             x[u] = SI ? madq(w, (jp >> (4 * d)) & 15u, x[u]) : x[u] + w;
         }
     }
@@ -125,36 +123,50 @@ __device__ __forceinline__ void sqa_reg_items(uint32_t *sw, const void *entv, in
     for (int u = 0; u < U; ++u) {
         const uint32_t a4 = (~(own[u] ^ up[u]) & M) + (~(own[u] ^ dn[u]) & M);
         // k = dE/2 + bias per byte: 2x + bias - deg + h for b_i = 0, its mirror 2 bias - that for b_i = 1
-        const uint32_t a = x[u] + x[u] + c0;
+        // (E = 2: four times that)
+        const uint32_t a = E == 2 ? 8u * x[u] + c0 : x[u] + x[u] + c0;
         const uint32_t b = K.k2 - a;
         const uint32_t m = own[u] * 0xFFu;
         const uint32_t kk = (a & ~m) | (b & m);
         const uint32_t full = SI ? 0u : a4 * K.W + kk;  // entry a W + k per byte, <= 3W - 1 <= 255
         const uint4 r4 = philox_sqa(iw[u], K.start, K.k1, K.L1, K.HA, K.LA, K.k0w, K.k1w, Kr);
         const uint32_t ur[4] = {r4.x, r4.y, r4.z, r4.w};
-        uint32_t rej = 0;
+        uint32_t bits = 0;  // E = 0: rejected replicas, else accepted ones
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            // u + entry carries into bit 32 exactly when the move is rejected
             const uint32_t sel = 0x4440u | (uint32_t)r;
+            if (E == 2) {
+                const uint32_t top = lds(__byte_perm(full, row, 0x7650u | (uint32_t)r));
+                asm("{ .reg .pred p; setp.le.u32 p, %1, %2; @p add.u32 %0, %0, %3; }"
+                    : "+r"(bits)
+                    : "r"(ur[r]), "r"(top), "r"(1u << (8 * r)));
+                continue;
+            }
             const uint32_t e = SI ? madq(__byte_perm(a4, 0u, sel), K.W, __byte_perm(kk, 0u, sel))
                                   : __byte_perm(full, 0u, sel);
-            const unsigned long long v = E32 ? (unsigned long long)static_cast<const uint32_t *>(entv)[e]
-                                             : static_cast<const unsigned long long *>(entv)[e];
-            rej |= (uint32_t)(((unsigned long long)ur[r] + v) >> 32) << (8 * r);
+            if (E == 1) {
+                const uint32_t top = lds(row + 4u * e);
+                asm("{ .reg .pred p; setp.le.u32 p, %1, %2; @p add.u32 %0, %0, %3; }"
+                    : "+r"(bits)
+                    : "r"(ur[r]), "r"(top), "r"(1u << (8 * r)));
+            } else {
+                // u + entry carries into bit 32 exactly when the move is rejected
+                const uint2 v = lds2(row + 8u * e);
+                bits |= (uint32_t)(((unsigned long long)ur[r] + ((unsigned long long)v.y << 32 | v.x)) >> 32) << (8 * r);
+            }
         }
-        nw[u] = own[u] ^ rej ^ M;  // flip where not rejected
+        nw[u] = own[u] ^ bits ^ (E == 0 ? M : 0u);  // flip where accepted
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        sts_q(sw, oa[u], nw[u]);
-        sts_q(sw, oa[u] + K.inv4, nw[u] ^ M);
+        sts(oa[u], nw[u]);
+        sts(oa[u] + K.inv4, nw[u] ^ M);
     }
 }
 
 // One parity pass of one colour-class slot: slices two at a time.
-template <int PAR, int MAXD, bool E32, bool SI>
-__device__ __forceinline__ void sqa_reg_pass(uint32_t *sw, const void *ent, int g, int G, int P, uint32_t own4,
+template <int PAR, int MAXD, int E, bool SI>
+__device__ __forceinline__ void sqa_reg_pass(uint32_t sw4, uint32_t row, int g, int G, int P, uint32_t own4,
                                              const uint32_t (&o4)[MAXD], uint32_t c0, uint32_t jp, uint32_t ib,
                                              const SqaRegConsts &K, const PhiloxKeys<2> &Kr)
 {
@@ -163,26 +175,26 @@ __device__ __forceinline__ void sqa_reg_pass(uint32_t *sw, const void *ent, int 
     const bool chain = G == 1;
     const uint32_t step = (uint32_t)dt * K.ns4, istep = (uint32_t)dt << 16;
     int tau = PAR + 2 * g;
-    uint32_t base = (uint32_t)tau * K.ns4;
+    uint32_t base = sw4 + (uint32_t)tau * K.ns4;
     uint32_t iw = ib | ((uint32_t)tau << 16);
     uint32_t prev_up = 0u;
     bool have = false;
     for (; tau + dt < P; tau += 2 * dt, base += 2 * step, iw += 2 * istep) {
         const int t2[2] = {tau, tau + dt};
         const uint32_t b2[2] = {base, base + step}, i2[2] = {iw, iw + istep};
-        sqa_reg_items<PAR, MAXD, 2, E32, SI>(sw, ent, P, t2, b2, i2, own4, o4, c0, jp, K, Kr, chain, have,
+        sqa_reg_items<PAR, MAXD, 2, E, SI>(row, P, t2, b2, i2, own4, o4, c0, jp, K, Kr, chain, have,
                                              prev_up);
         have = true;
     }
     if (tau < P) {
         const int t1[1] = {tau};
         const uint32_t b1[1] = {base}, i1[1] = {iw};
-        sqa_reg_items<PAR, MAXD, 1, E32, SI>(sw, ent, P, t1, b1, i1, own4, o4, c0, jp, K, Kr, chain, have,
+        sqa_reg_items<PAR, MAXD, 1, E, SI>(row, P, t1, b1, i1, own4, o4, c0, jp, K, Kr, chain, have,
                                              prev_up);
     }
 }
 
-template <bool PM1, int B, int MAXD, int NC, bool E32, bool SI>
+template <bool PM1, int B, int MAXD, int NC, int E, bool SI>
 __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad, uint32_t *smem)
 {
     const int tid = threadIdx.x;
@@ -196,20 +208,22 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
     const size_t Pn = (size_t)P * ns;
 
     unsigned long long *rows = reinterpret_cast<unsigned long long *>(smem);  // [2][3W]
-    uint32_t *sw = smem + 2 * 2 * 3 * (size_t)W;                            // [P][n + 1] plain
+    constexpr bool REG = NC > 0;  // the register form keeps a spin's data in registers
+    uint32_t *sw = smem + sqa_row_words(W, REG);                            // [P][n + 1] plain
     uint32_t *swi = sw + (PM1 ? Pn : 0);                                     // [P][n + 1] inverted
     uint32_t *meta_s = sw + (PM1 ? 2 * Pn : Pn);                             // [n]
     uint32_t *idx_s = meta_s + n;                                            // [n]
     uint16_t *off = reinterpret_cast<uint16_t *>(idx_s + n);                 // [MAXD][n] (+-1)
-    int *e2 = reinterpret_cast<int *>(idx_s + n + (PM1 ? ((size_t)MAXD * n + 1) / 2 : 0));
+    int *e2 = reinterpret_cast<int *>(REG ? meta_s : idx_s + n + (PM1 ? ((size_t)MAXD * n + 1) / 2 : 0));
     int *s_best = e2 + 4 * P;
     __shared__ int s_cptr[kMaxColours + 1];
 
     for (int c = tid; c <= ncol; c += B) s_cptr[c] = pr->cptr[c];
-    for (int p = tid; p < n; p += B) {
-        meta_s[p] = pr->meta[p];
-        idx_s[p] = (uint32_t)pr->idx_of_pos[p];
-    }
+    if (!REG)
+        for (int p = tid; p < n; p += B) {
+            meta_s[p] = pr->meta[p];
+            idx_s[p] = (uint32_t)pr->idx_of_pos[p];
+        }
     // initial state: top bit of the word at the initial-state slot, per slice
     for (size_t x = tid; x < Pn; x += B) {
         const int tau = (int)(x / ns), p = (int)(x - (size_t)tau * ns);
@@ -225,7 +239,7 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
         }
         sw[x] = w;
     }
-    if (PM1) {
+    if (PM1 && !REG) {
         for (int x = tid; x < MAXD * n; x += B) {
             const int d = x / n, p = x - d * n;
             uint16_t o = (uint16_t)n;  // missing neighbour: the slice's zero word
@@ -236,7 +250,7 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
             off[x] = o;
         }
     }
-    if (T > 0)
+    if (T > 0 && !REG)
         for (int x = tid; x < 3 * W; x += B) rows[x] = L.ent[x];
     __syncthreads();
 
@@ -247,11 +261,9 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
     const PhiloxKeys<2> Kr = philox_keys<2>(k0, k1);
 
     const int nt = (P > 1) ? P / 2 : 1;  // slices per parity
-    // register form: +-1 couplers, two or more slices, at most NC colour classes of at most B spins
-    bool reg = NC > 0 && PM1 && P > 1 && ncol <= NC;
-    for (int c = 0; reg && c < ncol; ++c) reg = s_cptr[c + 1] - s_cptr[c] <= B;
-    if constexpr (PM1 && NC > 0) {
-      if (reg) {
+    // register form: two or more slices, at most NC colour classes of at most B spins (the host's choice
+    // of this kernel covers every problem of the launch; reductions only shrink classes)
+    if constexpr (REG) {
         constexpr int NCR = NC;
         // class j: units (spin k, slice group g) = thread k + g nc, g < G = min(nt, B / nc)
         uint32_t own4[NCR], o4[NCR][MAXD], c0[NCR], ib[NCR], jp[NCR];
@@ -269,11 +281,19 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
                     G[j] = min(nt, B / nc);
                     if (tid < nc * G[j]) {
                         const int gq = tid / nc, p = lo + (tid - gq * nc);
-                        const uint32_t meta = meta_s[p];
+                        const uint32_t meta = pr->meta[p];
                         g[j] = gq;
                         own4[j] = 4u * (uint32_t)p;
 #pragma unroll
-                        for (int d = 0; d < MAXD; ++d) o4[j][d] = 4u * (uint32_t)off[d * n + p];
+                        for (int d = 0; d < MAXD; ++d) {
+                            // the inverted copy for J < 0, the slice's zero word for a missing neighbour
+                            uint32_t o = (uint32_t)n;
+                            if (d < (int)(meta & 0xFFFFu)) {
+                                const uint32_t e = pr->ell[(size_t)d * cap_n + p];
+                                o = ((e >> 31) ? (uint32_t)Pn : 0u) + (e & 0xFFFFu);
+                            }
+                            o4[j][d] = 4u * o;
+                        }
                         // bias - sum_j |J_ij| + h per byte (every |J| = 1: bias - deg + h)
                         int sumj = (int)(meta & 0xFFFFu);
                         if (SI) {
@@ -284,8 +304,8 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
                                 sumj += (int)aj;
                             }
                         }
-                        c0[j] = (uint32_t)(bias - sumj + ((int)meta >> 16)) * 0x01010101u;
-                        ib[j] = idx_s[p];
+                        c0[j] = (uint32_t)((E == 2 ? 4 : 1) * (bias - sumj + ((int)meta >> 16))) * 0x01010101u;
+                        ib[j] = (uint32_t)pr->idx_of_pos[p];
                     }
                 }
             }
@@ -294,44 +314,41 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
         K.ns4 = 4u * (uint32_t)ns;
         K.inv4 = 4u * (uint32_t)Pn;
         K.wrap4 = (uint32_t)(P - 1) * K.ns4;
-        K.k2 = (uint32_t)(2 * bias) * 0x01010101u;
-        K.W = (uint32_t)W;
+        K.k2 = (uint32_t)((E == 2 ? 8 : 2) * bias) * 0x01010101u;
+        K.W = (uint32_t)(E == 2 ? 4 * W : W);
         K.start = job.start;
         K.k1 = k1;
         K.L1 = L1;
         K.k0w = k0w;
         K.k1w = k1w;
-        // E32: the rows as 32-bit entries (low words) in the same space
-        uint32_t *rows32 = reinterpret_cast<uint32_t *>(rows);
-        if (E32) {
-            __syncthreads();  // every thread has read the 64-bit row 0
-            for (int x = tid; x < 3 * W; x += B) rows32[x] = (uint32_t)L.ent[x];
-            __syncthreads();
-        }
-        for (int t = 0; t < T; ++t) {
-            const void *ent = E32 ? static_cast<const void *>(rows32 + (t & 1) * 3 * W)
-                                  : static_cast<const void *>(rows + (t & 1) * 3 * W);
-            if (t + 1 < T) {
-                const unsigned long long *src = L.ent + (size_t)(t + 1) * 3 * W;
-                if (E32)
-                    for (int x = tid; x < 3 * W; x += B) rows32[((t + 1) & 1) * 3 * W + x] = (uint32_t)src[x];
-                else
-                    for (int x = tid; x < 3 * W; x += B) rows[((t + 1) & 1) * 3 * W + x] = src[x];
+        // rows of this and the next sweep: E > 0 in 32-bit words, the largest word accepted
+        uint32_t *rows32 = smem;
+        const int rstep = E == 2 ? 64 : 3 * W;
+        auto stage = [&](int t) {
+            const unsigned long long *src = L.ent + (size_t)t * 3 * W;
+            for (int x = tid; x < 3 * W; x += B) {
+                if (E > 0) rows32[(t & 1) * rstep + x] = ~(uint32_t)src[x];
+                else rows[(t & 1) * 3 * W + x] = src[x];
             }
+        };
+        if (T > 0) stage(0);
+        __syncthreads();
+        const uint32_t sw4 = shared_addr(sw), row4 = shared_addr(smem);
+        for (int t = 0; t < T; ++t) {
+            const uint32_t row = row4 + (uint32_t)(t & 1) * (E > 0 ? 4u * (uint32_t)rstep : 24u * (uint32_t)W);
+            if (t + 1 < T) stage(t + 1);
             philox_mulhilo(kPhiloxM0, H1 ^ (phase_hi | (uint32_t)t) ^ k0, K.HA, K.LA);
 #pragma unroll
             for (int j = 0; j < NCR; ++j) {
                 if (j < ncol) {
-                    sqa_reg_pass<0, MAXD, E32, SI>(sw, ent, g[j], G[j], P, own4[j], o4[j], c0[j], jp[j], ib[j], K, Kr);
+                    sqa_reg_pass<0, MAXD, E, SI>(sw4, row, g[j], G[j], P, own4[j], o4[j], c0[j], jp[j], ib[j], K, Kr);
                     __syncthreads();
-                    sqa_reg_pass<1, MAXD, E32, SI>(sw, ent, g[j], G[j], P, own4[j], o4[j], c0[j], jp[j], ib[j], K, Kr);
+                    sqa_reg_pass<1, MAXD, E, SI>(sw4, row, g[j], G[j], P, own4[j], o4[j], c0[j], jp[j], ib[j], K, Kr);
                     __syncthreads();
                 }
             }
         }
-      }
-    }
-    if (!reg)
+    } else
     for (int t = 0; t < T; ++t) {
         const unsigned long long *ent = rows + (t & 1) * 3 * W;
         if (t + 1 < T)
@@ -420,7 +437,7 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
         const int tau = (int)(x / n), p = (int)(x - (size_t)tau * n);
         const uint32_t *s = sw + (size_t)tau * ns;
         int c2[4];
-        energy2<PM1 && !SI>(s[p], meta_s[p], pr->ell, cap_n, p, s, c2);
+        energy2<PM1 && !SI>(s[p], REG ? pr->meta[p] : meta_s[p], pr->ell, cap_n, p, s, c2);
 #pragma unroll
         for (int r = 0; r < 4; ++r) atomicAdd(&e2[4 * tau + r], c2[r]);
     }
@@ -452,18 +469,31 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
     }
 }
 
-// NC > 0: register form for problems of at most NC colour classes of at most
-// B spins (+-1 couplers, two or more slices); other items take the walk.
-template <bool PM1, int B, int MAXD, int NC, bool E32, bool SI>
-__global__ void __launch_bounds__(B, (NC > 0 && B == 256) ? 2 : 1) k_sweep_sqa(const SweepLaunch L)
+// Resident CTAs per SM asked of the register allocator.  The 256-thread register form for
+// two colour classes and degree 6 fits three (80 registers, no spills; shared memory allows
+// three because the spins' data stays out of it), the other 256-thread forms two.
+// Chimera C8, 10 starts x (500 + 500), 16 slices, 500 sweeps: 46.5 ms with two CTAs and
+// carries of u + entry, 44.6 ms with three, one comparison per replica and the row's
+// address merged by the byte permute; the two integer pipes bound it (18 wide multiplies
+// and about 50 ALU instructions per four-replica item).
+template <int B, int MAXD, int NC, bool SI>
+constexpr int sqa_min_blocks()
 {
-    extern __shared__ __align__(16) uint32_t smem_sqa[];
+    return NC > 0 && B == 256 ? (NC == 2 && !SI && MAXD == 6 ? 3 : 2) : 1;
+}
+
+// NC > 0: register form for problems of at most NC colour classes of at most
+// B spins (+-1 or small integer couplers, two or more slices); 0: the item walk.
+template <bool PM1, int B, int MAXD, int NC, int E, bool SI>
+__global__ void __launch_bounds__(B, sqa_min_blocks<B, MAXD, NC, SI>()) k_sweep_sqa(const SweepLaunch L)
+{
+    extern __shared__ __align__(256) uint32_t smem_sqa[];
     __shared__ int s_item;
     for (int iter = 0;; ++iter) {
         SweepJob job;
         int quad0, nq;
         if (!next_item(L, iter, &s_item, job, quad0, nq)) break;
-        run_item_sqa<PM1, B, MAXD, NC, E32, SI>(L, job, quad0, smem_sqa);
+        run_item_sqa<PM1, B, MAXD, NC, E, SI>(L, job, quad0, smem_sqa);
         __syncthreads();
     }
 }
@@ -473,7 +503,7 @@ __global__ void __launch_bounds__(B, (NC > 0 && B == 256) ? 2 : 1) k_sweep_sqa(c
 // ent32, 32-bit acceptance entries; 3: the register form for small integer
 // couplers (|J| <= 15; block 256).  +-1 and small integers: neighbour
 // loop unrolled to MAXD (6 or 8).
-void *select_sqa(int variant, int block, int maxdeg, int ncls, bool ent32)
+void *select_sqa(int variant, int block, int maxdeg, int ncls, int e)
 {
 #define SPVAR_SQA_CASE(PM, BB, MD, NCC, E, S) \
     if (block == BB) return reinterpret_cast<void *>(k_sweep_sqa<PM, BB, MD, NCC, E, S>);
@@ -483,32 +513,31 @@ void *select_sqa(int variant, int block, int maxdeg, int ncls, bool ent32)
 #define SPVAR_SQA_SI(MD, NCC, E) SPVAR_SQA_CASE(true, 256, MD, NCC, E, true)
     const int md = maxdeg <= 6 ? 6 : maxdeg <= 8 ? 8 : 0;
     if (variant == 0) {
-        SPVAR_SQA_CASE(false, 128, 0, 0, false, false) SPVAR_SQA_CASE(false, 256, 0, 0, false, false)
-        SPVAR_SQA_CASE(false, 512, 0, 0, false, false)
+        SPVAR_SQA_CASE(false, 128, 0, 0, 0, false) SPVAR_SQA_CASE(false, 256, 0, 0, 0, false)
+        SPVAR_SQA_CASE(false, 512, 0, 0, 0, false)
     } else if (variant == 1 && md == 6) {
-        SPVAR_SQA_CASE(true, 128, 6, 0, false, false) SPVAR_SQA_CASE(true, 256, 6, 0, false, false)
-        SPVAR_SQA_CASE(true, 512, 6, 0, false, false)
+        SPVAR_SQA_CASE(true, 128, 6, 0, 0, false) SPVAR_SQA_CASE(true, 256, 6, 0, 0, false)
+        SPVAR_SQA_CASE(true, 512, 6, 0, 0, false)
     } else if (variant == 1 && md == 8) {
-        SPVAR_SQA_CASE(true, 128, 8, 0, false, false) SPVAR_SQA_CASE(true, 256, 8, 0, false, false)
-        SPVAR_SQA_CASE(true, 512, 8, 0, false, false)
+        SPVAR_SQA_CASE(true, 128, 8, 0, 0, false) SPVAR_SQA_CASE(true, 256, 8, 0, 0, false)
+        SPVAR_SQA_CASE(true, 512, 8, 0, 0, false)
     } else if (variant == 2) {
-        if (md == 6 && ncls == 2 && !ent32) { SPVAR_SQA_REG(6, 2, false) }
-        if (md == 6 && ncls == 2 && ent32) { SPVAR_SQA_REG(6, 2, true) }
-        if (md == 6 && ncls == 4 && !ent32) { SPVAR_SQA_REG(6, 4, false) }
-        if (md == 6 && ncls == 4 && ent32) { SPVAR_SQA_REG(6, 4, true) }
-        if (md == 8 && ncls == 2 && !ent32) { SPVAR_SQA_REG(8, 2, false) }
-        if (md == 8 && ncls == 2 && ent32) { SPVAR_SQA_REG(8, 2, true) }
-        if (md == 8 && ncls == 4 && !ent32) { SPVAR_SQA_REG(8, 4, false) }
-        if (md == 8 && ncls == 4 && ent32) { SPVAR_SQA_REG(8, 4, true) }
+#define SPVAR_SQA_E(MD, NCC)                            \
+    if (md == MD && ncls == NCC) {                      \
+        if (e == 2) { SPVAR_SQA_REG(MD, NCC, 2) }       \
+        if (e == 1) { SPVAR_SQA_REG(MD, NCC, 1) }       \
+        SPVAR_SQA_REG(MD, NCC, 0)                       \
+    }
+        SPVAR_SQA_E(6, 2) SPVAR_SQA_E(6, 4) SPVAR_SQA_E(8, 2) SPVAR_SQA_E(8, 4)
+#undef SPVAR_SQA_E
     } else if (variant == 3) {
-        if (md == 6 && ncls == 2 && !ent32) { SPVAR_SQA_SI(6, 2, false) }
-        if (md == 6 && ncls == 2 && ent32) { SPVAR_SQA_SI(6, 2, true) }
-        if (md == 6 && ncls == 4 && !ent32) { SPVAR_SQA_SI(6, 4, false) }
-        if (md == 6 && ncls == 4 && ent32) { SPVAR_SQA_SI(6, 4, true) }
-        if (md == 8 && ncls == 2 && !ent32) { SPVAR_SQA_SI(8, 2, false) }
-        if (md == 8 && ncls == 2 && ent32) { SPVAR_SQA_SI(8, 2, true) }
-        if (md == 8 && ncls == 4 && !ent32) { SPVAR_SQA_SI(8, 4, false) }
-        if (md == 8 && ncls == 4 && ent32) { SPVAR_SQA_SI(8, 4, true) }
+#define SPVAR_SQA_E(MD, NCC)                            \
+    if (md == MD && ncls == NCC) {                      \
+        if (e > 0) { SPVAR_SQA_SI(MD, NCC, 1) }         \
+        SPVAR_SQA_SI(MD, NCC, 0)                        \
+    }
+        SPVAR_SQA_E(6, 2) SPVAR_SQA_E(6, 4) SPVAR_SQA_E(8, 2) SPVAR_SQA_E(8, 4)
+#undef SPVAR_SQA_E
     }
 #undef SPVAR_SQA_SI
 #undef SPVAR_SQA_REG
@@ -516,11 +545,14 @@ void *select_sqa(int variant, int block, int maxdeg, int ncls, bool ent32)
     return nullptr;
 }
 
+// Form of the acceptance rows (see sqa_reg_items).
+int sqa_entries(bool ent32, int W) { return !ent32 ? 0 : 3 * W <= 64 ? 2 : 1; }
+
 }  // namespace
 
 bool sqa_shape_ok(int variant, int block, int max_n, int max_deg, int P, int W, int ncls)
 {
-    if (!select_sqa(variant, block, max_deg, ncls, false) || P < 1 || (P > 1 && (P & 1)) || P > kSqaMaxSlices) return false;
+    if (!select_sqa(variant, block, max_deg, ncls, 0) || P < 1 || (P > 1 && (P & 1)) || P > kSqaMaxSlices) return false;
     if (variant >= 2 && P < 2) return false;
     if ((long long)max_n >= (1 << 16) - 1) return false;
     if (variant != 0 && (long long)P * (max_n + 1) + max_n >= 0xFFFF) return false;
@@ -530,15 +562,15 @@ bool sqa_shape_ok(int variant, int block, int max_n, int max_deg, int P, int W, 
     return true;
 }
 
-size_t sqa_smem_bytes(int max_n, int P, int maxdeg, int W, bool pm1)
+size_t sqa_smem_bytes(int max_n, int P, int maxdeg, int W, int variant)
 {
-    return 4 * sqa_words(max_n, P, maxdeg, W, pm1);
+    return 4 * sqa_words(max_n, P, maxdeg, W, variant != 0, variant >= 2);
 }
 
 cudaError_t launch_sweep_sqa(const SweepLaunch &L, int variant, int block, int ncls, bool ent32, int grid,
                              size_t smem, cudaStream_t st)
 {
-    void *k = select_sqa(variant, block, L.max_deg, ncls, ent32);
+    void *k = select_sqa(variant, block, L.max_deg, ncls, sqa_entries(ent32, L.W));
     if (!k) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -546,9 +578,9 @@ cudaError_t launch_sweep_sqa(const SweepLaunch &L, int variant, int block, int n
     return cudaLaunchKernel(k, dim3(grid), dim3(block), args, smem, st);
 }
 
-int sqa_max_active_blocks(int variant, int block, int max_deg, int ncls, bool ent32, size_t smem)
+int sqa_max_active_blocks(int variant, int block, int max_deg, int ncls, int W, bool ent32, size_t smem)
 {
-    void *k = select_sqa(variant, block, max_deg, ncls, ent32);
+    void *k = select_sqa(variant, block, max_deg, ncls, sqa_entries(ent32, W));
     if (!k) return 0;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int nb = 0;
