@@ -738,15 +738,10 @@ int spvar_reduce(const spvar_problem *p, const int8_t *fixed, int32_t *old_of_ne
     Problem *D = new (std::nothrow) Problem();
     if (!D) return SPVAR_ENOMEM;
     D->device = S->device;
-    D->blob_bytes = prob_blob_bytes(H.cap_n, H.cap_nnz, H.maxdeg);
-    int32_t *scratch = nullptr;
+    // one allocation: the fold's scratch behind the problem's arrays
+    const size_t prob_bytes = prob_blob_bytes(H.cap_n, H.cap_nnz, H.maxdeg);
+    D->blob_bytes = prob_bytes + 4 * slot_scratch_ints(H.cap_n);
     if (cudaMalloc(&D->blob, D->blob_bytes) != cudaSuccess) {
-        delete D;
-        cudaGetLastError();
-        return SPVAR_ENOMEM;
-    }
-    if (cudaMalloc(&scratch, 8 * (size_t)H.cap_n) != cudaSuccess) {
-        cudaFree(D->blob);
         delete D;
         cudaGetLastError();
         return SPVAR_ENOMEM;
@@ -754,15 +749,14 @@ int spvar_reduce(const spvar_problem *p, const int8_t *fixed, int32_t *old_of_ne
     std::memset(&D->hdr, 0, sizeof(DevProb));
     prob_carve(&D->hdr, D->blob, H.cap_n, H.cap_nnz, H.maxdeg);
     D->dev = static_cast<DevProb *>(D->blob);
+    int32_t *scratch = reinterpret_cast<int32_t *>(static_cast<char *>(D->blob) + prob_bytes);
     cudaStream_t st = as_stream(stream);
-    bool ok = cudaMemcpyAsync(D->dev, &D->hdr, sizeof(DevProb), cudaMemcpyHostToDevice, st) == cudaSuccess;
-    if (ok) ok = launch_reduce_single(S->dev, D->dev, fixed, old_of_new, scratch, st) == cudaSuccess;
+    bool ok = launch_reduce_single(S->dev, D->dev, D->hdr, fixed, old_of_new, scratch, st) == cudaSuccess;
     DevProb back;
-    if (ok) ok = cudaMemcpyAsync(&back, D->dev, sizeof(DevProb), cudaMemcpyDeviceToHost, st) == cudaSuccess;
-    if (ok) ok = cudaStreamSynchronize(st) == cudaSuccess;
     int32_t cptr[kMaxColours + 1] = {0};
-    if (ok) ok = cudaMemcpy(cptr, back.cptr, sizeof(int32_t) * (back.ncol + 1), cudaMemcpyDeviceToHost) == cudaSuccess;
-    cudaFree(scratch);
+    if (ok) ok = cudaMemcpyAsync(&back, D->dev, sizeof(DevProb), cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    if (ok) ok = cudaMemcpyAsync(cptr, D->hdr.cptr, sizeof(cptr), cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    if (ok) ok = cudaStreamSynchronize(st) == cudaSuccess;
     if (!ok) {
         cudaFree(D->blob);
         delete D;

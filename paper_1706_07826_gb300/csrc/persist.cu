@@ -280,13 +280,6 @@ __global__ void __launch_bounds__(kCountBlock)
     count_bs_core(P, spins, W, elite, k, canon, fix_num, fix_den, counts, fixed, nfixed, nullptr, nullptr, blockIdx.x, sm);
 }
 
-__global__ void __launch_bounds__(kBigBlock) k_reduce_single(const DevProb *src, DevProb *dst,
-                                                             const int8_t *fixed,
-                                                             int32_t *old_of_new, int32_t *scratch)
-{
-    reduce_core(src, dst, fixed, old_of_new, scratch);
-}
-
 // ----------------------------------------------------------- multi-start slots
 __global__ void __launch_bounds__(256) k_slots_init(Slot *slots, SolveConsts C)
 {
@@ -757,7 +750,8 @@ constexpr int kScanCols = 6;  // colour classes ranked per multi-value scan
 // Chunks ch[0..CB) of the CTA (-1: none).  The spins' own values and the
 // table of chunk totals are loaded once for all of them, so the chunks' scans
 // follow one another without a global load in between.
-template <int CB>
+// ORIG: the original index of every free spin is carried along.
+template <int CB, bool ORIG = true>
 __device__ __forceinline__ void fold_index(Slot &s, const int (&ch)[CB])
 {
     __shared__ int s_w[32 * (2 + kScanCols)];
@@ -785,7 +779,7 @@ __device__ __forceinline__ void fold_index(Slot &s, const int (&ch)[CB])
         rc[b] = valid[b] ? rowcnt[i] : 0;
         colv[b] = valid[b] ? P->colour[i] : -1;
         h[b] = valid[b] ? hfold[i] : 0;
-        oi[b] = valid[b] ? orig[i] : 0;
+        oi[b] = ORIG && valid[b] ? orig[i] : 0;
     }
     // offsets of each chunk (totals of the chunks before it) and the totals of all:
     // field f (0 free spins, 1 free-free entries, 2 + c spins of class c) summed by a warp
@@ -881,7 +875,7 @@ __device__ __forceinline__ void fold_index(Slot &s, const int (&ch)[CB])
         if (valid[b]) npos[i] = f[b] ? (uint32_t)a | ((uint32_t)pos << 16) : ~0u;
         if (f[b]) {
             oon[a] = i;
-            orig2[a] = oi[b];
+            if (ORIG) orig2[a] = oi[b];
             dh[a] = h[b];
             dcolour[a] = col;
             drow[a] = s_base[b][1] + exr;
@@ -971,6 +965,57 @@ __device__ __forceinline__ void fold_fill(Slot &s, const int (&ch)[G])
                 ++d[g];
             }
     }
+}
+
+// The fold and compaction of one problem by a cluster; the caller's barrier
+// stands before it and, where the result is read on, after it.
+template <bool ORIG>
+__device__ __forceinline__ void fold_cluster(Slot &s, int n, int rank)
+{
+    const int nch = max(1, (n + kFoldChunk - 1) / kFoldChunk);
+    // this CTA's chunks rank, rank + kPassCluster, ..., two at a time in the gather stages
+    for (int c = rank; c < nch; c += 2 * kPassCluster) {
+        const int ch[2] = {c, c + kPassCluster < nch ? c + kPassCluster : -1};
+        fold_count<2>(s, ch);
+    }
+    pass_barrier();
+    for (int c = rank; c < nch; c += kIndexBatch * kPassCluster) {
+        int ch[kIndexBatch];
+#pragma unroll
+        for (int b = 0; b < kIndexBatch; ++b) ch[b] = c + b * kPassCluster < nch ? c + b * kPassCluster : -1;
+        fold_index<kIndexBatch, ORIG>(s, ch);
+    }
+    pass_barrier();
+    for (int c = rank; c < nch; c += 2 * kPassCluster) {
+        const int ch[2] = {c, c + kPassCluster < nch ? c + kPassCluster : -1};
+        fold_fill<2>(s, ch);
+    }
+}
+
+// The standalone reduction: the pass's fold stages on one cluster.  Bound by
+// the latency of its dependent gathers, which one CTA of 1024 threads walked
+// through a spin at a time.
+__global__ void __cluster_dims__(kPassCluster, 1, 1) __launch_bounds__(kPassBlock)
+    k_reduce_single(const DevProb *src, DevProb *dst, DevProb hdr, const int8_t *fixed,
+                    int32_t *old_of_new, int32_t *scratch)
+{
+    Slot s;
+    s.cur = const_cast<DevProb *>(src);
+    s.next = 0;
+    s.buf[0] = dst;
+    s.ocur = 0;
+    s.orig[0] = s.orig[1] = nullptr;
+    s.fixed = const_cast<int8_t *>(fixed);
+    s.old_of_new = old_of_new;
+    s.scratch = scratch;
+    const int rank = blockIdx.x;
+    if (rank == 0 && threadIdx.x == 0) {
+        *dst = hdr;  // capacities and arrays; the fold fills in the sizes
+        *reinterpret_cast<unsigned long long *>(scratch + fold_table_offset(hdr.cap_n) +
+                                                kFoldMaxChunks * kFoldStride) = 0ull;
+    }
+    pass_barrier();
+    fold_cluster<false>(s, src->n, rank);
 }
 
 // Dynamic shared memory of the pass: the elite list (Smax entries), then one
@@ -1091,24 +1136,7 @@ __global__ void __cluster_dims__(kPassCluster, 1, 1) __launch_bounds__(kPassBloc
         }
         pass_barrier();
     }
-    const int nch = max(1, (n + kFoldChunk - 1) / kFoldChunk);
-    // this CTA's chunks rank, rank + kPassCluster, ..., two at a time in the gather stages
-    for (int c = rank; c < nch; c += 2 * kPassCluster) {
-        const int ch[2] = {c, c + kPassCluster < nch ? c + kPassCluster : -1};
-        fold_count<2>(s, ch);
-    }
-    pass_barrier();
-    for (int c = rank; c < nch; c += kIndexBatch * kPassCluster) {
-        int ch[kIndexBatch];
-#pragma unroll
-        for (int b = 0; b < kIndexBatch; ++b) ch[b] = c + b * kPassCluster < nch ? c + b * kPassCluster : -1;
-        fold_index<kIndexBatch>(s, ch);
-    }
-    pass_barrier();
-    for (int c = rank; c < nch; c += 2 * kPassCluster) {
-        const int ch[2] = {c, c + kPassCluster < nch ? c + kPassCluster : -1};
-        fold_fill<2>(s, ch);
-    }
+    fold_cluster<true>(s, n, rank);
     pass_barrier();
     // 4. the phase transition
     if (rank == 0 && tid == 0) {
@@ -1350,10 +1378,10 @@ cudaError_t launch_count_single(const DevProb *prob, int n_host, const uint32_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_single(const DevProb *src, DevProb *dst, const int8_t *fixed,
+cudaError_t launch_reduce_single(const DevProb *src, DevProb *dst, const DevProb &hdr, const int8_t *fixed,
                                  int32_t *old_of_new, int32_t *scratch, cudaStream_t stream)
 {
-    k_reduce_single<<<1, kBigBlock, 0, stream>>>(src, dst, fixed, old_of_new, scratch);
+    k_reduce_single<<<kPassCluster, kPassBlock, 0, stream>>>(src, dst, hdr, fixed, old_of_new, scratch);
     return cudaGetLastError();
 }
 

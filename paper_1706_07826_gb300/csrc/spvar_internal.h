@@ -531,7 +531,9 @@ cudaError_t launch_elite_single(const int64_t *energies, int S, int k, int32_t *
 cudaError_t launch_count_single(const DevProb *prob, int n_host, const uint32_t *spins, int W,
                                 const int32_t *elite, int k, int canon, int fix_num, int fix_den,
                                 int32_t *counts, int8_t *fixed, int32_t *nfixed, cudaStream_t stream);
-cudaError_t launch_reduce_single(const DevProb *src, DevProb *dst, const int8_t *fixed,
+// Fold and compact src into dst, whose capacities and arrays `hdr` holds; scratch
+// of slot_scratch_ints(cap_n) ints.
+cudaError_t launch_reduce_single(const DevProb *src, DevProb *dst, const DevProb &hdr, const int8_t *fixed,
                                  int32_t *old_of_new, int32_t *scratch, cudaStream_t stream);
 int elite_max_samples();
 
