@@ -294,7 +294,7 @@ int spvar_reduce(const spvar_problem *p, const int8_t *fixed, int32_t *old_of_ne
  * every device allocation and forbids allocating calls after start-up).  It
  * computes the same reduction as spvar_reduce but allocates nothing: the
  * result goes to caller buffers as plain CSR, and the working arrays live in
- * a static device array of 2 * SPVAR_NOALLOC_MAX_N int32 (128 KB) that every
+ * a static device array of SPVAR_NOALLOC_MAX_N int32 (64 KB) that every
  * device loading the library keeps until the process exits.
  *   fixed            device int8 [n] (0, +1, -1)
  *   row_ptr          device [n+1] out (first n'+1 entries written)

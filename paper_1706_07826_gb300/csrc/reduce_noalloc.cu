@@ -17,15 +17,19 @@
 // streams, or concurrent host threads) race on it and must be serialised by
 // the caller.  Nothing in the array needs to start at zero: each call writes
 // every entry it later reads.
+#include <cooperative_groups.h>
+
 #include <mutex>
 
 #include "persist.cuh"
 
+namespace cg = cooperative_groups;
+
 namespace spvar {
 namespace {
 
-// new index of every old spin, then the free-free row lengths: 2 x n ints
-__device__ __align__(256) int32_t g_reduce_scratch[2 * SPVAR_NOALLOC_MAX_N];
+// new index of every old spin (-1: fixed)
+__device__ __align__(256) int32_t g_reduce_scratch[SPVAR_NOALLOC_MAX_N];
 
 std::mutex g_addr_mu;
 int32_t *g_addr[64] = {nullptr};
@@ -47,90 +51,141 @@ int scratch_address(int32_t **out)
     return SPVAR_OK;
 }
 
+constexpr int kCsrCluster = 8;  // blocks, each with a contiguous range of the spins
+constexpr int kCsrSpins = (SPVAR_NOALLOC_MAX_N + kCsrCluster * kBigBlock - 1) / (kCsrCluster * kBigBlock);
+constexpr int kCsrGather = 4;   // CSR entries of a row loaded at once
+
+struct CsrTotals {
+    int32_t nfree, nnz;
+    unsigned long long off;
+};
+
 // Fold the fixed spins into h and the offset and write the CSR of the free
-// spins (renumbered in increasing old index) to the caller's arrays.  One
-// 1024-thread CTA.
-__global__ void __launch_bounds__(kBigBlock)
+// spins (renumbered in increasing old index) to the caller's arrays.
+// Bound by the latency of the dependent gathers (spin, row, neighbour), so the
+// spins are dealt to the blocks of one cluster and a thread holds its own
+// (at most kCsrSpins) in registers; the blocks exchange their totals through
+// shared memory, and only the new indices go through the scratch array.
+// 8000 spins of a cubic lattice: 61.7 us a call on one block, 14.6 here.
+__global__ void __cluster_dims__(kCsrCluster, 1, 1) __launch_bounds__(kBigBlock)
     k_reduce_csr(const DevProb *S, const int8_t *fixed, int32_t *row_ptr, int32_t *col, int32_t *val,
                  int32_t *h_out, int64_t *offset_out, int32_t *old_of_new, int32_t *n_out, int32_t *scratch)
 {
     __shared__ int s_warp[32];
-    __shared__ unsigned long long s_off;
-    const int tid = threadIdx.x, B = blockDim.x;
-    const int n = S->n;
-    int32_t *new_of_old = scratch;
-    int32_t *rowcnt = scratch + SPVAR_NOALLOC_MAX_N;
-    if (tid == 0) s_off = 0ull;
+    __shared__ CsrTotals s_tot;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int tid = threadIdx.x, rank = blockIdx.x;
+    const int n = S->n, len = (n + kCsrCluster - 1) / kCsrCluster;
+    const int first = rank * len, last = min(n, first + len);
+    const int32_t *srow = S->row_ptr, *scol = S->col, *sval = S->val;
+    if (tid == 0) s_tot.off = 0ull;
     __syncthreads();
 
-    int carry = 0;
-    for (int base = 0; base < n; base += B) {
-        const int i = base + tid;
-        const int f = (i < n && fixed[i] == 0) ? 1 : 0;
-        int tot;
-        const int ex = block_scan_excl(f, s_warp, &tot);
-        if (i < n) {
-            new_of_old[i] = f ? carry + ex : -1;
-            if (f) old_of_new[carry + ex] = i;
-        }
-        carry += tot;
-    }
-    const int m = carry;
-    __syncthreads();
-
-    long long off_part = 0;
-    for (int i = tid; i < n; i += B) {
-        const int vi = fixed[i];
-        long long hf = S->h[i];
-        int nfree = 0;
-        for (int p = S->row_ptr[i]; p < S->row_ptr[i + 1]; ++p) {
-            const int j = S->col[p];
-            const int vj = fixed[j];
-            if (vi) {
-                if (vj && j > i) off_part += (long long)S->val[p] * vi * vj;
-            } else {
-                if (vj) hf += (long long)S->val[p] * vj;
-                else ++nfree;
+    // folded biases, free-free row lengths, and their sums over the spins before, by block
+    int32_t hf[kCsrSpins], a[kCsrSpins], q[kCsrSpins];
+    bool fr[kCsrSpins];
+    long long off = 0;
+    int nfree = 0, nnz = 0;
+#pragma unroll
+    for (int u = 0; u < kCsrSpins; ++u) {
+        const int i = first + u * kBigBlock + tid;
+        const bool ok = i < last;
+        const int vi = ok ? fixed[i] : 0, h = ok ? S->h[i] : 0;
+        const int p0 = ok ? srow[i] : 0, p1 = ok ? srow[i + 1] : 0;
+        long long hs = h;
+        int cnt = 0;
+        for (int p = p0; p < p1; p += kCsrGather) {
+            int j[kCsrGather], v[kCsrGather], f[kCsrGather];
+#pragma unroll
+            for (int d = 0; d < kCsrGather; ++d) {
+                j[d] = p + d < p1 ? scol[p + d] : -1;
+                v[d] = p + d < p1 ? sval[p + d] : 0;
+            }
+#pragma unroll
+            for (int d = 0; d < kCsrGather; ++d) f[d] = j[d] >= 0 ? fixed[j[d]] : 0;
+#pragma unroll
+            for (int d = 0; d < kCsrGather; ++d) {
+                if (j[d] < 0) continue;
+                if (vi) {
+                    if (f[d] && j[d] > i) off += (long long)v[d] * vi * f[d];
+                } else if (f[d]) {
+                    hs += (long long)v[d] * f[d];
+                } else {
+                    ++cnt;
+                }
             }
         }
-        if (vi) {
-            off_part += (long long)S->h[i] * vi;
-        } else {
-            const int a = new_of_old[i];
-            h_out[a] = (int32_t)hf;
-            rowcnt[a] = nfree;
-        }
-    }
-    atomicAdd(&s_off, (unsigned long long)off_part);
-    __syncthreads();
-
-    carry = 0;
-    for (int base = 0; base < m; base += B) {
-        const int a = base + tid;
-        const int c = (a < m) ? rowcnt[a] : 0;
+        if (vi) off += (long long)h * vi;
+        fr[u] = ok && !vi;
+        hf[u] = (int32_t)hs;
         int tot;
-        const int ex = block_scan_excl(c, s_warp, &tot);
-        if (a < m) row_ptr[a] = carry + ex;
-        carry += tot;
+        a[u] = nfree + block_scan_excl(fr[u] ? 1 : 0, s_warp, &tot);
+        nfree += tot;
+        q[u] = nnz + block_scan_excl(fr[u] ? cnt : 0, s_warp, &tot);
+        nnz += tot;
     }
-    if (tid == 0) row_ptr[m] = carry;
-    __syncthreads();
-
-    for (int a = tid; a < m; a += B) {
-        const int i = old_of_new[a];
-        int q = row_ptr[a];
-        for (int p = S->row_ptr[i]; p < S->row_ptr[i + 1]; ++p) {
-            const int j = S->col[p];
-            if (fixed[j] == 0) {
-                col[q] = new_of_old[j];
-                val[q] = S->val[p];
-                ++q;
-            }
-        }
-    }
+#pragma unroll
+    for (int sh = 16; sh > 0; sh >>= 1) off += __shfl_xor_sync(0xFFFFFFFFu, off, sh);
+    if ((tid & 31) == 0) atomicAdd(&s_tot.off, (unsigned long long)off);
     if (tid == 0) {
+        s_tot.nfree = nfree;
+        s_tot.nnz = nnz;
+    }
+    cluster.sync();  // every block's totals
+
+    int base_n = 0, base_z = 0, m = 0, z = 0;
+    unsigned long long osum = 0ull;
+    for (int r = 0; r < kCsrCluster; ++r) {
+        const CsrTotals *t = cluster.map_shared_rank(&s_tot, r);
+        if (r < rank) {
+            base_n += t->nfree;
+            base_z += t->nnz;
+        }
+        m += t->nfree;
+        z += t->nnz;
+        osum += t->off;
+    }
+    if (rank == 0 && tid == 0) {
+        row_ptr[m] = z;
         *n_out = m;
-        *offset_out = S->offset + (long long)s_off;
+        *offset_out = S->offset + (long long)osum;
+    }
+#pragma unroll
+    for (int u = 0; u < kCsrSpins; ++u) {
+        const int i = first + u * kBigBlock + tid;
+        a[u] += base_n;
+        q[u] += base_z;
+        if (i < last) scratch[i] = fr[u] ? a[u] : -1;
+        if (fr[u]) {
+            old_of_new[a[u]] = i;
+            h_out[a[u]] = hf[u];
+            row_ptr[a[u]] = q[u];
+        }
+    }
+    cluster.sync();  // the new indices, and no block leaves while its totals are read
+
+#pragma unroll
+    for (int u = 0; u < kCsrSpins; ++u) {
+        const int i = first + u * kBigBlock + tid;
+        const int p0 = fr[u] ? srow[i] : 0, p1 = fr[u] ? srow[i + 1] : 0;
+        int w = q[u];
+        for (int p = p0; p < p1; p += kCsrGather) {
+            int j[kCsrGather], v[kCsrGather];
+#pragma unroll
+            for (int d = 0; d < kCsrGather; ++d) {
+                j[d] = p + d < p1 ? scol[p + d] : -1;
+                v[d] = p + d < p1 ? sval[p + d] : 0;
+            }
+#pragma unroll
+            for (int d = 0; d < kCsrGather; ++d) j[d] = j[d] >= 0 ? scratch[j[d]] : -1;
+#pragma unroll
+            for (int d = 0; d < kCsrGather; ++d)
+                if (j[d] >= 0) {
+                    col[w] = j[d];
+                    val[w] = v[d];
+                    ++w;
+                }
+        }
     }
 }
 
@@ -158,7 +213,7 @@ extern "C" int spvar_reduce_noalloc(const spvar_problem *p, const int8_t *fixed,
     const DevProb *src = S->dev;
     void *args[] = {(void *)&src, (void *)&fixed, (void *)&row_ptr, (void *)&col, (void *)&val, (void *)&h,
                     (void *)&offset, (void *)&old_of_new, (void *)&n_out, (void *)&scratch};
-    const cudaError_t e = cudaLaunchKernel(reinterpret_cast<const void *>(k_reduce_csr), dim3(1), dim3(kBigBlock),
-                                           args, 0, reinterpret_cast<cudaStream_t>(stream));
+    const cudaError_t e = cudaLaunchKernel(reinterpret_cast<const void *>(k_reduce_csr), dim3(kCsrCluster),
+                                           dim3(kBigBlock), args, 0, reinterpret_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? SPVAR_OK : SPVAR_ECUDA;
 }

@@ -1,8 +1,9 @@
 """GPU parity of the clustered fold behind spvar.reduce at the edges of its
 256-spin chunks: one spin, a chunk less and more by one spin, all eight blocks
 of the cluster with one and with several chunks, and the largest problem, with
-few and with most spins fixed.  The sweep layout is compared through the
-energies of a sample of the reduced problem."""
+few and with most spins fixed, the sweep layout compared through the energies of
+a sample of the reduced problem; and of the allocation-free form at the edges of
+the eight blocks' ranges and of a thread's first and second spin."""
 import numpy as np
 import pytest
 
@@ -25,6 +26,29 @@ def _ring(n, seed):
     J = g.integers(1, 8, len(ei)) * (g.integers(0, 2, len(ei)) * 2 - 1)
     return I.Instance("ring", n, ei.astype(np.int32), ej.astype(np.int32), J.astype(np.int32),
                       g.integers(-5, 6, n).astype(np.int32))
+
+
+@pytest.mark.parametrize("free", [0.0, 0.15, 0.8])
+@pytest.mark.parametrize("n", [1, 2, 7, 9, 1025, 8191, 8192, 8193, 16384])
+def test_reduce_noalloc_equals_oracle_at_block_edges(cuda_lib, n, free):
+    import torch
+    spvar = cuda_lib
+    inst = _ring(n, 900 + n)
+    g = np.random.default_rng(n + 1)
+    fixed = np.where(g.random(n) < free, 0, g.choice([-1, 1], n)).astype(np.int8)
+    red, _, oon = O.reduce(oracle_problem(inst), fixed)
+    gp = gpu_problem(inst)
+    z = {k: torch.full((max(s, 1),), -9, dtype=t, device="cuda")
+         for k, s, t in (("row_ptr", n + 1, torch.int32), ("col", 2 * inst.m, torch.int32),
+                         ("val", 2 * inst.m, torch.int32), ("h", n, torch.int32), ("offset", 1, torch.int64),
+                         ("old_of_new", n, torch.int32), ("n_out", 1, torch.int32))}
+    spvar.reduce_noalloc(gp, torch.from_numpy(fixed).cuda(), **z)
+    d = {k: v.cpu().numpy() for k, v in z.items()}
+    m, nnz = red.n, int(red.row_ptr[red.n])
+    assert d["n_out"][0] == m and d["offset"][0] == red.offset
+    assert np.array_equal(d["row_ptr"][:m + 1], red.row_ptr)
+    for k, want, cnt in (("col", red.col, nnz), ("val", red.val, nnz), ("h", red.h, m), ("old_of_new", oon, m)):
+        assert np.array_equal(d[k][:cnt], want[:cnt]) and (d[k][cnt:] == -9).all(), k
 
 
 @pytest.mark.parametrize("free", [0.15, 0.8])
