@@ -510,8 +510,13 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
     SweepShape sh{0, (H.n >= 512) ? 256 : 128, Q, 1, 0, 0};
     if (pm1_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
         const int md = H.maxdeg <= 6 ? 6 : 8;
+        // 256 threads, unless 128 hold the classes in as many slots (a warp without items anneals
+        // dummy words): 500 sweeps, 3D L = 4, 64 to 5000 samples 221 .. 469 us at 256, 135 .. 288 at
+        // 128; L = 5, 1300 samples 870 against 435.  Where a class then takes two slots, 256
+        // stay (Chimera C8, 1000 samples, 1000 sweeps: 620 us at 256, 735 at 128).
+        const bool small = pm1_nslot(P, Q, 128) == pm1_nslot(P, Q, 256);
         if (pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg))
-            for (int blk : {256, 512, 128}) {
+            for (int blk : {small ? 128 : 256, 256, 512, 128}) {
                 const int ns = pm1_nslot(P, Q, blk);
                 if (ns > 0 && pm1_shape_ok(blk, ns, md, 0)) { sh = SweepShape{1, blk, Q, 0, ns, md}; break; }
             }

@@ -299,7 +299,10 @@ __device__ void run_item_pm1(const SweepLaunch &L, const SweepJob &job, int quad
     // colour-aligned slots
     SlotRegs<MAXD> s[NSLOT];
     uint32_t barmask = 0;
-    const RoundKeys K = philox_keys<3>(k0, k1);
+    RoundKeys K;
+    // small integer couplers: 2.7 % faster with the keys formed behind the slots (U_10 Chimera C8, 2000
+    // samples, 1000 sweeps: 1538 -> 1497 us); the byte-lane forms up to 14 % slower
+    if (!SI) K = philox_keys<3>(k0, k1);
     const uint32_t dummy = 4u * (uint32_t)(KW - 1), zero = 4u * (uint32_t)(2 * KW);
 #pragma unroll
     for (int j = 0; j < NSLOT; ++j) {
@@ -358,6 +361,7 @@ __device__ void run_item_pm1(const SweepLaunch &L, const SweepJob &job, int quad
             }
         }
     }
+    if (SI) K = philox_keys<3>(k0, k1);
     const uint32_t k16 = SCALED ? (uint32_t)(32 * bias) * 0x00010001u : (uint32_t)(16 * bias) * 0x01010101u;
     const uint32_t *thr = L.thr;
     const size_t ts = (size_t)L.thr_stride;
@@ -405,10 +409,233 @@ __global__ void __launch_bounds__(B, (pm1_min_blocks<B, NSLOT, MAXD, SCALED>()))
     }
 }
 
+// ------------------------------------------------------------ latency form
+// The byte-lane kernel for a grid that leaves the chip mostly empty (a few
+// short anneals): its time is then the chain of one warp, whose half-sweep
+// holds ten Philox rounds in program order between the barrier and the
+// acceptance.  Here B more threads compute the random numbers, and the
+// acceptance rows, of KA sweeps ahead into shared memory, and the sweeping
+// threads are left with load, sum, look-up, store and their barrier.  The warp
+// schedulers they share are idle most of the time.  Warps without an item of
+// any class take no part, and a lone sweeping warp needs no barrier at all.
+// Computing the next sweep's numbers in the same thread instead was 7 %
+// slower: the instructions still issue in the order of one warp.
+constexpr int kAheadMax = 8;       // sweeps of one buffer at most
+constexpr int kAheadPer = 2;       // threads that run ahead per sweeping thread
+constexpr int kAheadWords = 1024;  // random words (of 16 bytes) of one buffer
+template <int B, int NSLOT>
+struct Pm1AheadSmem {
+    static constexpr int KW = B * NSLOT + 1;
+    unsigned long long row[2][kAheadMax][kRowE];  // 256 bytes each, aligned: entry offsets merge into the address
+    uint4 u[2][kAheadWords];                      // by sweep, slot and thread
+    uint32_t sw[2 * KW + 1];
+    int cptr[kMaxColours + 1];
+};
+
+// How a block's threads share an item: `act` sweeping threads (whole warps),
+// `groups` times as many that run ahead (group g the sweeps g, g + groups, ...
+// of a buffer), and `ka` sweeps a buffer.
+struct AheadSplit {
+    int act, groups, ka;
+    __device__ int threads() const { return act * (1 + groups); }
+};
+
+// Named barriers of k_sweep_pm1_ahead (0 is the block's own).
+constexpr int kBarSweep = 1, kBarFull = 2, kBarEmpty = 4;
+__device__ __forceinline__ void bar_sync(int id, int threads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// The items of thread tid: slots filled class by class, as in run_item_pm1.
+// Returns the slots that begin a colour class other than the first as a bit mask.
+template <int B, int NSLOT, int MAXD>
+__device__ __forceinline__ uint32_t ahead_slots(const DevProb *P, const SweepJob &job, int quad0, int nq,
+                                                const Pm1AheadSmem<B, NSLOT> &sm, int tid, int bias,
+                                                SlotRegs<MAXD> (&s)[NSLOT])
+{
+    constexpr int KW = Pm1AheadSmem<B, NSLOT>::KW;
+    const int n = P->n, ncol = P->ncol, cap_n = P->cap_n;
+    uint32_t barmask = 0;
+    int c = 0, jb = 0;  // class of slot j, its first slot
+#pragma unroll
+    for (int j = 0; j < NSLOT; ++j) {
+        // without an item: the dummy word, zero neighbours
+        s[j].own = 4u * (uint32_t)(KW - 1);
+#pragma unroll
+        for (int d = 0; d < MAXD; ++d) s[j].nb[d] = 4u * (uint32_t)(2 * KW);
+        s[j].c0 = (uint32_t)(8 * bias) * 0x01010101u;
+        s[j].A = s[j].L0k = s[j].D = s[j].H3k = s[j].L3 = 0u;
+        while (c < ncol && j >= jb + ((sm.cptr[c + 1] - sm.cptr[c]) * nq + B - 1) / B) {
+            jb += ((sm.cptr[c + 1] - sm.cptr[c]) * nq + B - 1) / B;
+            ++c;
+        }
+        if (c >= ncol) continue;
+        const int nc = sm.cptr[c + 1] - sm.cptr[c], local = (j - jb) * B + tid;
+        if (j == jb && j > 0) barmask |= 1u << j;
+        if (local >= nc * nq) continue;
+        const int q = local / nc, p = sm.cptr[c] + (local - q * nc);
+        const uint32_t meta = P->meta[p];
+        const int deg = (int)(meta & 0xFFFFu), h = (int)meta >> 16;
+        s[j].own = 4u * (uint32_t)(q * n + p);
+#pragma unroll
+        for (int d = 0; d < MAXD; ++d)
+            if (d < deg) {
+                const uint32_t e = P->ell[(size_t)d * cap_n + p];
+                s[j].nb[d] = 4u * (uint32_t)(((e >> 31) ? KW : 0) + q * n + (int)(e & 0xFFFFu));
+            }
+        s[j].c0 = (uint32_t)(8 * (bias - deg + h)) * 0x01010101u;
+        philox_setup(s[j], (uint32_t)P->idx_of_pos[p], (uint32_t)(quad0 + q), job.start, (uint32_t)job.seed,
+                     (uint32_t)(job.seed >> 32));
+    }
+    return barmask;
+}
+
+// The random numbers and rows of sweeps t0 .. T - 1; x: the thread among those that run ahead.
+template <int B, int NSLOT, int MAXD>
+__device__ __forceinline__ void ahead_produce(Pm1AheadSmem<B, NSLOT> &sm, const SlotRegs<MAXD> (&s)[NSLOT], int x,
+                                              const AheadSplit &sp, int t0, int T, uint32_t phase_hi,
+                                              const RoundKeys &K, const uint32_t *thr, size_t ts, int bias)
+{
+    const int grp = x / sp.act, lane = x - grp * sp.act, all = sp.act * sp.groups;
+    constexpr int kRows = kAheadMax * kRowE / 32;
+    int buf = 0;
+    for (int t = t0; t < T; t += sp.ka, buf ^= 1) {
+        // the rows' entries are loaded first and stored last
+        uint32_t e[kRows];
+#pragma unroll
+        for (int c = 0; c < kRows; ++c) {
+            const int y = x + c * all, k = y / kRowE, i = y % kRowE - bias;
+            e[c] = (k < sp.ka && i > 0 && i <= bias && t + k < T) ? __ldg(thr + (size_t)(t + k) * ts + 2 * i) : 0u;
+        }
+        if (t >= t0 + 2 * sp.ka) bar_sync(kBarEmpty + buf, sp.threads());
+        for (int k = grp; k < sp.ka && t + k < T; k += sp.groups)
+#pragma unroll
+            for (int j = 0; j < NSLOT; ++j)
+                sm.u[buf][(k * NSLOT + j) * sp.act + lane] = philox_slot(s[j], phase_hi | (uint32_t)(t + k), K);
+#pragma unroll
+        for (int c = 0; c < kRows; ++c) {
+            const int y = x + c * all, k = y / kRowE, i = y % kRowE - bias;
+            if (k < sp.ka) sm.row[buf][k][y % kRowE] = i > 0 && i <= bias ? (1ull << 32) - e[c] : 0ull;
+        }
+        bar_arrive(kBarFull + buf, sp.threads());
+    }
+}
+
+// ONE: a single sweeping warp.
+template <int B, int NSLOT, int MAXD, bool ONE>
+__device__ __forceinline__ void ahead_sweep(Pm1AheadSmem<B, NSLOT> &sm, const SlotRegs<MAXD> (&s)[NSLOT], int tid,
+                                            const AheadSplit &sp, int t0, int T, uint32_t barmask, uint32_t k16)
+{
+    const int act = ONE ? 32 : sp.act, threads = sp.threads();
+    constexpr uint32_t kInv = 4u * (uint32_t)Pm1AheadSmem<B, NSLOT>::KW;
+    const uint32_t base = shared_addr(sm.sw);
+    auto sync = [&] {
+        if (ONE) __syncwarp();
+        else bar_sync(kBarSweep, act);
+    };
+    // a spin's word is changed by its own thread only
+    uint32_t own[NSLOT];
+#pragma unroll
+    for (int j = 0; j < NSLOT; ++j) own[j] = lds(base + s[j].own);
+    int buf = 0;
+    for (int t = t0; t < T; t += sp.ka, buf ^= 1) {
+        bar_sync(kBarFull + buf, threads);
+        const int kt = min(sp.ka, T - t);
+        for (int k = 0; k < kt; ++k) {
+            const uint32_t row = shared_addr(sm.row[buf][k]), ua = shared_addr(&sm.u[buf][k * NSLOT * act + tid]);
+#pragma unroll
+            for (int j = 0; j < NSLOT; ++j) {
+                if (ONE ? j > 0 : (barmask & (1u << j)) != 0) sync();
+                uint32_t nbw[MAXD];
+#pragma unroll
+                for (int d = 0; d < MAXD; ++d) nbw[d] = lds(base + s[j].nb[d]);
+                const uint4 u = lds4(ua + 16u * (uint32_t)(act * j));  // behind the neighbours: it is needed last
+                uint32_t x = nbw[0];
+#pragma unroll
+                for (int d = 1; d < MAXD; ++d) x += nbw[d];
+                const uint32_t a = (x << 4) + s[j].c0, m = own[j] * 0xFFu;
+                const uint32_t idx8 = (a & ~m) | ((k16 - a) & m);
+                const uint32_t ur[4] = {u.x, u.y, u.z, u.w};
+                uint32_t c[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint2 e = lds2(__byte_perm(idx8, row, 0x7650u | (uint32_t)r));
+                    c[r] = (uint32_t)(((unsigned long long)ur[r] + ((unsigned long long)e.y << 32 | e.x)) >> 32);
+                }
+                const uint32_t inv = own[j] ^ ((c[0] + (c[1] << 8)) + ((c[2] + (c[3] << 8)) << 16));
+                own[j] = inv ^ 0x01010101u;
+                sts(base + s[j].own, own[j]);
+                sts(base + s[j].own + kInv, inv);
+            }
+            sync();
+        }
+        if (t + 2 * sp.ka < T) bar_arrive(kBarEmpty + buf, threads);
+    }
+}
+
+template <int B, int NSLOT, int MAXD>
+__global__ void __launch_bounds__((1 + kAheadPer) * B) k_sweep_pm1_ahead(const SweepLaunch L)
+{
+    __shared__ __align__(256) Pm1AheadSmem<B, NSLOT> sm;
+    __shared__ int s_item;
+    constexpr int KW = Pm1AheadSmem<B, NSLOT>::KW;
+    const bool sweeper = (int)threadIdx.x < B;
+    for (int iter = 0;; ++iter) {
+        SweepJob job;
+        int quad0, nq;
+        if (!next_item(L, iter, &s_item, job, quad0, nq)) break;
+        const DevProb *P = job.prob;
+        const int n = P->n, ncol = P->ncol, bias = P->dmax >> 1;
+        for (int c = threadIdx.x; c <= ncol; c += blockDim.x) sm.cptr[c] = P->cptr[c];
+        init_spins(P, job, quad0, nq, sm.sw, sm.sw + KW);
+        if (threadIdx.x == 0) sm.sw[KW - 1] = sm.sw[2 * KW - 1] = sm.sw[2 * KW] = 0u;
+        __syncthreads();
+        AheadSplit sp;
+        sp.act = 32;
+        for (int c = 0; c < ncol; ++c) sp.act = max(sp.act, ((sm.cptr[c + 1] - sm.cptr[c]) * nq + 31) & ~31);
+        sp.act = min(sp.act, B);
+        sp.ka = min(kAheadMax, kAheadWords / (NSLOT * sp.act));
+        sp.groups = min(kAheadPer * B / sp.act, sp.ka);
+        const int x = (int)threadIdx.x - (sweeper ? 0 : B);
+        SlotRegs<MAXD> s[NSLOT];
+        const uint32_t barmask = ahead_slots<B, NSLOT, MAXD>(P, job, quad0, nq, sm, x % sp.act, bias, s);
+        const int T = job_end(L, job);
+        const uint32_t k16 = (uint32_t)(16 * bias) * 0x01010101u;
+        if (!sweeper) {
+            if (x < sp.act * sp.groups)
+                ahead_produce<B, NSLOT, MAXD>(sm, s, x, sp, job.t0, T, job.phase << kSweepBits, philox_keys<3>((uint32_t)job.seed, (uint32_t)(job.seed >> 32)),
+                                              L.thr, (size_t)L.thr_stride, bias);
+        } else if (x < sp.act) {
+            if (sp.act == 32)
+                ahead_sweep<B, NSLOT, MAXD, true>(sm, s, x, sp, job.t0, T, barmask, k16);
+            else
+                ahead_sweep<B, NSLOT, MAXD, false>(sm, s, x, sp, job.t0, T, barmask, k16);
+        }
+        __syncthreads();
+        finish_item<true>(P, job, quad0, nq, sm.sw, reinterpret_cast<int *>(sm.sw + KW));
+        __syncthreads();
+    }
+}
+
 template <int B, int NSLOT, int MAXD, bool SCALED, bool SI>
 void *kernel_ptr()
 {
     return reinterpret_cast<void *>(k_sweep_pm1<B, NSLOT, MAXD, SCALED, SI>);
+}
+
+void *select_ahead(int block, int nslot, int maxd)
+{
+#define SPVAR_AHEAD_CASE(BB, NS, MD) \
+    if (block == BB && nslot == NS && maxd == MD) return reinterpret_cast<void *>(k_sweep_pm1_ahead<BB, NS, MD>);
+    SPVAR_AHEAD_CASE(128, 2, 6) SPVAR_AHEAD_CASE(128, 3, 6) SPVAR_AHEAD_CASE(128, 4, 6)
+    SPVAR_AHEAD_CASE(128, 2, 8) SPVAR_AHEAD_CASE(128, 3, 8) SPVAR_AHEAD_CASE(128, 4, 8)
+#undef SPVAR_AHEAD_CASE
+    return nullptr;
 }
 
 void *select_kernel(int block, int nslot, int maxd, int mode)
@@ -466,6 +693,16 @@ cudaError_t launch_sweep_pm1(const SweepLaunch &L, int block, int nslot, int max
     SweepLaunch A = L;
     A.thr_stride = L.thr_step;
     void *args[] = {&A};
+    // a grid of at most one block per SM: the latency form.  1000 sweeps, +-1 couplers: 3D L = 4, 64 or
+    // 256 samples 349 -> 234 us; L = 5 649 -> 513; L = 6 363 -> 335; Chimera C3 352 -> 267, C5 357 -> 324.
+    // With two or three blocks per SM its extra threads get in the way (L = 6, 1500 samples, 375 blocks:
+    // 488 us without, 750 with), and with 256 sweeping threads the shared-memory pipe bounds
+    // both forms (L = 8, 300 samples: 447 without, 461 with), so only the 128-thread shapes have it.
+    void *ahead = scaled ? nullptr : select_ahead(block, nslot, maxd);
+    int dev = 0, sms = 0;
+    if (ahead && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && grid <= sms)
+        return cudaLaunchKernel(ahead, dim3(grid), dim3((1 + kAheadPer) * block), args, 0, st);
     return cudaLaunchKernel(k, dim3(grid), dim3(block), args, scaled ? smem : 0, st);
 }
 

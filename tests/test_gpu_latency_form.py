@@ -1,0 +1,52 @@
+"""GPU parity of the +-1 register kernel's latency form, which grids of at most
+one 128-thread block per SM take: one to four sweeping warps, two and three
+colour classes, degree 8, biases up to the widest byte-lane row, sweep counts
+around its buffers (none, one, part of one, several and a remainder), and a sample
+in two sweep ranges.  Everything is a whole number
+and equals the oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1706_07826_gb300 import instances as I
+
+from gpu_cases import gpu_problem, oracle_problem, table
+
+pytestmark = pytest.mark.gpu
+
+
+def _ring(n, offsets, seed, hmax):
+    """+-1 couplers to the given offsets of a ring."""
+    g = np.random.default_rng(seed)
+    ei = np.repeat(np.arange(n), len(offsets)).astype(np.int32)
+    ej = ((ei + np.tile(offsets, n)) % n).astype(np.int32)
+    J = (g.integers(0, 2, len(ei)) * 2 - 1).astype(np.int32)
+    return I.Instance("ring", n, ei, ej, J, g.integers(-hmax, hmax + 1, n).astype(np.int32))
+
+
+CASES = {
+    "one_warp": lambda: I.cubic3d(4, 801),
+    "one_warp_odd": lambda: I.cubic3d(3, 802),
+    "two_warps_three_classes": lambda: I.cubic3d(5, 803),
+    "four_warps": lambda: I.chimera(5, 804),
+    "few_spins": lambda: _ring(6, [1], 805, 2),
+    "degree8": lambda: _ring(62, [1, 3, 5, 9], 806, 7),
+}
+
+
+@pytest.mark.parametrize("T", [0, 1, 7, 8, 9, 16, 17, 37])
+@pytest.mark.parametrize("name", list(CASES))
+def test_sample_equals_oracle(cuda_lib, name, T):
+    spvar = cuda_lib
+    inst = CASES[name]()
+    S, seed = 22, 96
+    thr = table(inst, max(T, 1))[:T]
+    p, dev = gpu_problem(inst), spvar.thresholds_device(table(inst, max(T, 1)))
+    words, e = spvar.sample(p, dev, thr.shape[1], T, S, seed)
+    spins, energies, _ = O.sample(oracle_problem(inst), thr, S, seed)
+    assert np.array_equal(e.cpu().numpy()[:S], energies)
+    assert np.array_equal(spvar.unpack_spins(words.cpu().numpy()[:S], inst.n), spins)
+    cut = T // 3
+    half, _ = spvar.sample_range(p, dev, thr.shape[1], 0, cut, S, seed)
+    w2, e2 = spvar.sample_range(p, dev, thr.shape[1], cut, T, S, seed, init=half)
+    assert bool((e2 == e).all()) and bool((w2 == words).all())
