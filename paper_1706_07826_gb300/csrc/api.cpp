@@ -259,7 +259,9 @@ namespace {
 // kernel, whose threads take two spins at once without a set-up.  Measured, 500 sweeps: 3D L =
 // 12 with 250 quads 1.43 ms (1024 threads, pairs) against 1.69 streaming, with 100 quads
 // 1.13 against 0.98 streaming; L = 9 with 50 quads 1.09 against 1.35 streaming.
-SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, bool pm1)
+// *cost (if not null): the busiest SM's rounds per sweep, one of which takes about 0.15 n ns.
+SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, bool pm1,
+                            double *cost = nullptr)
 {
     const DevProb &H = P->hdr;
     const int md = H.maxdeg <= 6 ? 6 : 8;
@@ -297,12 +299,52 @@ SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int
                 best.Q = Q;
             }
         }
+    if (cost) *cost = best_t;
     if (pm1 && best.block > 0 && pm1s_shape_ok(512, md, H.n, 1)) {
         const int bytes = (int)pm1s_smem_bytes(H.n, 1, md) + (2 << 10), k = ceil_div(quads, sms);
         const int occ = std::min(optin / bytes, 2), conc = std::min(k, occ);
         double work = 0.0;
         for (int c = 0; c < H.ncol; ++c) work += 1.86 * ceil(P->csize[c] / 1024.0);
         if (occ > 0 && ceil((double)k / conc) * work * 4.0 * conc < best_t) best = SweepShape{2, 512, 1, 0, 0, md};
+    }
+    return best;
+}
+
+// Shape of one sample of `quads` quads on the byte-lane register kernel: the block size and
+// quads per item whose busiest SM is done first.  A slot (a colour class's spins of a block, with
+// dummy words on the threads left over) takes a warp 180 ns in a row (215 with several quads, which
+// share no Philox products; 110 in the latency form), and a scheduler 72 ns per warp (76 in blocks of
+// 512, whose barriers are wider); about 768 threads are resident, and the two bounds overlap in
+// part.  Measured, 400 sweeps, against 256 threads with quads / (2 SMs) quads each: 3D L = 4, 64
+// samples 183 -> 112 us; L = 6, 10000 samples 1871 -> 910; L = 8, 5000 samples 1933 -> 994;
+// Chimera C8, 4000 samples 1116 -> 781.
+SweepShape register_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, int md)
+{
+    SweepShape best{1, 0, 1, 0, 0, md};
+    double best_t = 1e300, best_work = 0.0;
+    for (int Q = 1; Q <= 8; ++Q)
+        for (int B : {128, 256, 512}) {
+            const int ns = pm1_nslot(P, Q, B);
+            if (ns == 0 || !pm1_shape_ok(B, ns, md, 0)) continue;
+            const int items = ceil_div(quads, Q), k = ceil_div(items, sms);
+            const double slot = B == 128 && items <= sms ? 110.0 : Q == 1 ? 180.0 : 215.0;
+            const double chain = std::max(k * B / 768.0, 1.0) * ns * slot, work = k * ns * (B / 128.0) * (B == 512 ? 76.0 : 72.0);
+            const double t = std::max(chain, work) + 0.2 * std::min(chain, work);
+            if (t < best_t) {
+                best_t = t;
+                best_work = work;
+                best.block = B;
+                best.Q = Q;
+                best.nslot = ns;
+            }
+        }
+    // Where large classes leave many threads of every slot over, and with several items per SM, the
+    // quad-group kernel is the faster one (Chimera C9, 324 spins a class in two slots of 256: 8000
+    // samples, 400 sweeps, 2885 -> 2536 us; 10000 samples, a last round of items nearly empty, stay).
+    if (best.block > 0 && quads >= 6 * sms && P->hdr.n >= 512) {
+        double rounds = 0.0;
+        const SweepShape g = quad_group_shape(P, quads, sms, optin, thr_stride, true, &rounds);
+        if (g.kind == 6 && g.block > 0 && 0.154 * P->hdr.n * rounds < 0.88 * best_work) return g;
     }
     return best;
 }
@@ -510,16 +552,10 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
     SweepShape sh{0, (H.n >= 512) ? 256 : 128, Q, 1, 0, 0};
     if (pm1_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
         const int md = H.maxdeg <= 6 ? 6 : 8;
-        // 256 threads, unless 128 hold the classes in as many slots (a warp without items anneals
-        // dummy words): 500 sweeps, 3D L = 4, 64 to 5000 samples 221 .. 469 us at 256, 135 .. 288 at
-        // 128; L = 5, 1300 samples 870 against 435.  Where a class then takes two slots, 256
-        // stay (Chimera C8, 1000 samples, 1000 sweeps: 620 us at 256, 735 at 128).
-        const bool small = pm1_nslot(P, Q, 128) == pm1_nslot(P, Q, 256);
-        if (pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg))
-            for (int blk : {small ? 128 : 256, 256, 512, 128}) {
-                const int ns = pm1_nslot(P, Q, blk);
-                if (ns > 0 && pm1_shape_ok(blk, ns, md, 0)) { sh = SweepShape{1, blk, Q, 0, ns, md}; break; }
-            }
+        if (pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
+            const SweepShape c = register_shape(P, quads, sms, optin, thr_stride, md);
+            if (c.block > 0) sh = c;
+        }
         // large problems: the quad-group kernel, or (large biases) the streaming one (one quad per CTA)
         if (sh.kind == 0 && pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
             const SweepShape c = quad_group_shape(P, quads, sms, optin, thr_stride, true);

@@ -50,3 +50,18 @@ def test_sample_equals_oracle(cuda_lib, name, T):
     half, _ = spvar.sample_range(p, dev, thr.shape[1], 0, cut, S, seed)
     w2, e2 = spvar.sample_range(p, dev, thr.shape[1], cut, T, S, seed, init=half)
     assert bool((e2 == e).all()) and bool((w2 == words).all())
+
+
+@pytest.mark.parametrize("name,S", [("one_warp", 2611), ("two_warps_three_classes", 4001), ("four_warps", 1300),
+                                    ("one_warp_odd", 16000), ("degree8", 5003), ("chimera9", 8002)])
+def test_sample_of_many_quads_equals_oracle(cuda_lib, name, S):
+    """Shapes of spvar_sample by the number of quads: several per block, a part
+    of the last block, and the quad-group kernel for Chimera C9."""
+    spvar = cuda_lib
+    inst = I.chimera(9, 807) if name == "chimera9" else CASES[name]()
+    T, seed = 3, 97
+    thr = table(inst, T)
+    words, e = spvar.sample(gpu_problem(inst), spvar.thresholds_device(thr), thr.shape[1], T, S, seed)
+    spins, energies, _ = O.sample(oracle_problem(inst), thr, S, seed)
+    assert np.array_equal(e.cpu().numpy()[:S], energies)
+    assert np.array_equal(spvar.unpack_spins(words.cpu().numpy()[:S], inst.n), spins)
