@@ -310,38 +310,44 @@ SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int
     return best;
 }
 
-// Shape of one sample of `quads` quads on the byte-lane register kernel: the block size and
-// quads per item whose busiest SM is done first.  A slot (a colour class's spins of a block, with
-// dummy words on the threads left over) takes a warp 180 ns in a row (215 with several quads, which
-// share no Philox products; 110 in the latency form), and a scheduler 72 ns per warp (76 in blocks of
-// 512, whose barriers are wider); about 768 threads are resident, and the two bounds overlap in
-// part.  Measured, 400 sweeps, against 256 threads with quads / (2 SMs) quads each: 3D L = 4, 64
-// samples 183 -> 112 us; L = 6, 10000 samples 1871 -> 910; L = 8, 5000 samples 1933 -> 994;
-// Chimera C8, 4000 samples 1116 -> 781.
-SweepShape register_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, int md)
+// Shape of one sample of `quads` quads on the register kernel (mode 0: byte lanes, 1 and 2: the
+// 16-bit lanes): the block size and quads per item whose busiest SM is done first.  A slot (a
+// colour class's spins of a block, with dummy words on the threads left over) takes a warp 180 ns
+// in a row (215 with several quads, which share no Philox products; 110 in the latency form), and a
+// scheduler 72 ns per warp (76 in blocks of 512, whose barriers are wider, 68 in those of 576, two
+// of which are resident); about 768 threads are resident (512 of the 16-bit lanes, which take about
+// half as long again for everything), and the two bounds overlap in part.  Measured, 400 sweeps,
+// against 256 threads with quads / (2 SMs) quads each: 3D L = 4, 64 samples 183 -> 112 us; L = 6,
+// 10000 samples 1871 -> 910; L = 8, 5000 samples 1933 -> 994; Chimera C8, 4000 samples 1116 -> 781;
+// and where that many quads did not fit four slots and the general kernel ran: U_10 C12, 2500 samples
+// 5211 -> 1662, weak-strong C10, 4000 samples 5804 -> 2306.
+SweepShape register_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, int md, int mode)
 {
-    SweepShape best{1, 0, 1, 0, 0, md};
+    SweepShape best{1, 0, 1, mode, 0, md};
     double best_t = 1e300, best_work = 0.0;
     for (int Q = 1; Q <= 8; ++Q)
-        for (int B : {128, 256, 512}) {
-            const int ns = pm1_nslot(P, Q, B);
-            if (ns == 0 || !pm1_shape_ok(B, ns, md, 0)) continue;
+        for (int B : {128, 256, 512, 576, 1024}) {
+            int ns = pm1_nslot(P, Q, B);
+            if (mode != 0 && (ns == 3 || (ns == 2 && !pm1_shape_ok(B, 2, md, mode)))) ns = 4;
+            if (ns == 0 || (mode == 0 && B > 512) || !pm1_shape_ok(B, ns, md, mode)) continue;
+            const SweepShape c{1, B, Q, mode, ns, md};
+            if (mode != 0 && sweep_shape_smem(c, P->hdr.n, thr_stride, P->hdr.maxdeg) > (size_t)optin) continue;
             const int items = ceil_div(quads, Q), k = ceil_div(items, sms);
-            const double slot = B == 128 && items <= sms ? 110.0 : Q == 1 ? 180.0 : 215.0;
-            const double chain = std::max(k * B / 768.0, 1.0) * ns * slot, work = k * ns * (B / 128.0) * (B == 512 ? 76.0 : 72.0);
+            const double slot = mode == 0 && B == 128 && items <= sms ? 110.0 : Q == 1 ? 180.0 : 215.0;
+            const double resident = mode == 0 ? 768.0 : B == 576 ? 1152.0 : B == 1024 ? 1024.0 : 512.0;
+            const double chain = std::max(k * B / resident, 1.0) * ns * slot;
+            const double work = k * ns * (B / 128.0) * (B == 576 ? 68.0 : B >= 512 ? 76.0 : 72.0);
             const double t = std::max(chain, work) + 0.2 * std::min(chain, work);
             if (t < best_t) {
                 best_t = t;
                 best_work = work;
-                best.block = B;
-                best.Q = Q;
-                best.nslot = ns;
+                best = c;
             }
         }
     // Where large classes leave many threads of every slot over, and with several items per SM, the
     // quad-group kernel is the faster one (Chimera C9, 324 spins a class in two slots of 256: 8000
     // samples, 400 sweeps, 2885 -> 2536 us; 10000 samples, a last round of items nearly empty, stay).
-    if (best.block > 0 && quads >= 6 * sms && P->hdr.n >= 512) {
+    if (mode == 0 && best.block > 0 && quads >= 6 * sms && P->hdr.n >= 512) {
         double rounds = 0.0;
         const SweepShape g = quad_group_shape(P, quads, sms, optin, thr_stride, true, &rounds);
         if (g.kind == 6 && g.block > 0 && 0.154 * P->hdr.n * rounds < 0.88 * best_work) return g;
@@ -553,7 +559,7 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
     if (pm1_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
         const int md = H.maxdeg <= 6 ? 6 : 8;
         if (pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
-            const SweepShape c = register_shape(P, quads, sms, optin, thr_stride, md);
+            const SweepShape c = register_shape(P, quads, sms, optin, thr_stride, md, 0);
             if (c.block > 0) sh = c;
         }
         // large problems: the quad-group kernel, or (large biases) the streaming one (one quad per CTA)
@@ -572,19 +578,13 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
         // one coupler magnitude per spin, or small integer couplers: the register
         // kernel's 16-bit-lane variants
         const int md = H.maxdeg <= 6 ? 6 : 8;
-        for (int blk : {256, 512, 576, 1024}) {
-            int ns = pm1_nslot(P, Q, blk);
-            if (ns == 3) ns = 4;
-            const SweepShape c{1, blk, Q, mode16, ns, md};
-            if (ns > 0 && pm1_shape_ok(blk, ns, md, mode16) &&
-                sweep_shape_smem(c, H.n, thr_stride, H.maxdeg) <= (size_t)optin) {
-                sh = c;
-                break;
-            }
-        }
+        const SweepShape c = register_shape(P, quads, sms, optin, thr_stride, md, mode16);
+        if (c.block > 0) sh = c;
     }
-    if (sh.kind == 0 && mode16 == 0 && H.maxdeg <= 8) {
-        // couplers of several magnitudes: the quad-group kernel for integer couplers
+    if (sh.kind == 0 && H.maxdeg <= 8) {
+        // couplers of several magnitudes, and problems too large for the 16-bit-lane register
+        // kernel: the quad-group kernel for integer couplers (400 sweeps, U_10 C18: 64 samples 2855 us on
+        // the general kernel, 1231 here; 4000 samples 17546 and 5334)
         const SweepShape c = quad_group_shape(P, quads, sms, optin, thr_stride, false);
         if (c.block > 0) sh = c;
     }

@@ -65,3 +65,20 @@ def test_sample_of_many_quads_equals_oracle(cuda_lib, name, S):
     spins, energies, _ = O.sample(oracle_problem(inst), thr, S, seed)
     assert np.array_equal(e.cpu().numpy()[:S], energies)
     assert np.array_equal(spvar.unpack_spins(words.cpu().numpy()[:S], inst.n), spins)
+
+
+@pytest.mark.parametrize("make,S", [(lambda: I.weak_strong(4, 808), 1300), (lambda: I.weak_strong(6, 809), 5002),
+                                    (lambda: I.chimera_u10(3, 810), 9999), (lambda: I.chimera_u10(8, 811), 2501),
+                                    (lambda: I.chimera_u10(18, 812), 30), (lambda: I.weak_strong(17, 813), 30)],
+                         ids=["ws4", "ws6", "u10_c3", "u10_c8", "u10_c18", "ws17"])
+def test_sample_of_16_bit_lanes_equals_oracle(cuda_lib, make, S):
+    """The same rule for the 16-bit-lane forms, and the quad-group kernel for
+    problems whose classes their blocks do not hold."""
+    spvar = cuda_lib
+    inst = make()
+    T, seed = 3, 98
+    thr = table(inst, T)
+    words, e = spvar.sample(gpu_problem(inst), spvar.thresholds_device(thr), thr.shape[1], T, S, seed)
+    spins, energies, _ = O.sample(oracle_problem(inst), thr, S, seed)
+    assert np.array_equal(e.cpu().numpy()[:S], energies)
+    assert np.array_equal(spvar.unpack_spins(words.cpu().numpy()[:S], inst.n), spins)
