@@ -556,20 +556,24 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
     const int optin = device_smem_optin();
     // shape: the register-resident +-1 kernel when it applies, else the general one
     SweepShape sh{0, (H.n >= 512) ? 256 : 128, Q, 1, 0, 0};
+    // the call's limit: the problem fits the shared memory of the general kernel at this Q or, +-1
+    // couplers, of the streaming one; the quad-group kernels' smaller footprint does not widen it
+    const bool general_fits =
+        sweep_shape_smem(SweepShape{0, sh.block, Q, 0, 0, 0}, H.n, thr_stride, H.maxdeg) <= (size_t)optin;
     if (pm1_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
         const int md = H.maxdeg <= 6 ? 6 : 8;
+        const bool streaming_fits =
+            pm1s_shape_ok(512, md, H.n, 1) && pm1s_smem_bytes(H.n, 1, md) <= (size_t)optin;
         if (pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
             const SweepShape c = register_shape(P, quads, sms, optin, thr_stride, md, 0);
             if (c.block > 0) sh = c;
         }
         // large problems: the quad-group kernel, or (large biases) the streaming one (one quad per CTA)
-        if (sh.kind == 0 && pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg)) {
+        if (sh.kind == 0 && pm1r_kernel_eligible(H.pm1 != 0, H.dmax, H.maxdeg) && (streaming_fits || general_fits)) {
             const SweepShape c = quad_group_shape(P, quads, sms, optin, thr_stride, true);
             if (c.block > 0) sh = c;
         }
-        if (sh.kind == 0 && pm1s_shape_ok(512, md, H.n, 1) &&
-            pm1s_smem_bytes(H.n, 1, md) <= (size_t)optin)
-            sh = SweepShape{2, 512, 1, 0, 0, md};
+        if (sh.kind == 0 && streaming_fits) sh = SweepShape{2, 512, 1, 0, 0, md};
     }
     const int mode16 = ujr_kernel_eligible(H.ujs != 0, H.dmax, H.maxdeg)          ? 1
                        : sir_kernel_eligible(P->jabs_max, H.dmax, H.maxdeg) ? 2
@@ -581,7 +585,7 @@ int spvar_sample_range(const spvar_problem *p, int32_t sweep_begin, int32_t swee
         const SweepShape c = register_shape(P, quads, sms, optin, thr_stride, md, mode16);
         if (c.block > 0) sh = c;
     }
-    if (sh.kind == 0 && H.maxdeg <= 8) {
+    if (sh.kind == 0 && H.maxdeg <= 8 && general_fits) {
         // couplers of several magnitudes, and problems too large for the 16-bit-lane register
         // kernel: the quad-group kernel for integer couplers (400 sweeps, U_10 C18: 64 samples 2855 us on
         // the general kernel, 1231 here; 4000 samples 17546 and 5334)

@@ -69,3 +69,15 @@ def test_sample_equals_oracle(cuda_lib, name):
     half, _ = spvar.sample_range(p, dev, thr.shape[1], 0, 5, S, seed)
     w2, e2 = spvar.sample_range(p, dev, thr.shape[1], 5, T, S, seed, init=half)
     assert bool((e2 == e).all()) and bool((w2 == words).all())
+
+
+def test_sample_limit_is_the_general_kernels(cuda_lib):
+    """A sample whose eight quads per block pass the general kernel's shared
+    memory is refused, although the quad-group kernel could hold it."""
+    spvar = cuda_lib
+    inst = _gauss(20, 608, 100)
+    thr = table(inst, 2)
+    p, dev = gpu_problem(inst), spvar.thresholds_device(thr)
+    with pytest.raises(spvar.SpvarError):
+        spvar.sample(p, dev, thr.shape[1], 2, 16000, 1)
+    spvar.sample(p, dev, thr.shape[1], 2, 40, 1)
