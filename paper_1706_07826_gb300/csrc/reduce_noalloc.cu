@@ -53,6 +53,7 @@ int scratch_address(int32_t **out)
 
 constexpr int kCsrCluster = 8;  // blocks, each with a contiguous range of the spins
 constexpr int kCsrSpins = (SPVAR_NOALLOC_MAX_N + kCsrCluster * kBigBlock - 1) / (kCsrCluster * kBigBlock);
+constexpr int kCsrOneBlock = kCsrSpins * kBigBlock;  // the most spins one block takes
 constexpr int kCsrGather = 4;   // CSR entries of a row loaded at once
 
 struct CsrTotals {
@@ -66,16 +67,24 @@ struct CsrTotals {
 // spins are dealt to the blocks of one cluster and a thread holds its own
 // (at most kCsrSpins) in registers; the blocks exchange their totals through
 // shared memory, and only the new indices go through the scratch array.
-// 8000 spins of a cubic lattice: 61.7 us a call on one block, 14.6 here.
-__global__ void __cluster_dims__(kCsrCluster, 1, 1) __launch_bounds__(kBigBlock)
-    k_reduce_csr(const DevProb *S, const int8_t *fixed, int32_t *row_ptr, int32_t *col, int32_t *val,
-                 int32_t *h_out, int64_t *offset_out, int32_t *old_of_new, int32_t *n_out, int32_t *scratch)
+// 8000 spins of a cubic lattice: 61.7 us a call on one block, 14.6 here.  Up
+// to kCsrOneBlock spins one block takes the same two spins a thread, and its
+// launch is 2 to 3 us cheaper for the host (elite, counts and this reduction
+// of Chimera C16, n = 2048: 64.4 us a call by the cluster, 57.5 by the block;
+// C19, n = 2888: 80.7 us by one block to the end on the device, 68.8 here).
+template <int NB>  // blocks
+__device__ __forceinline__ void reduce_csr(const DevProb *S, const int8_t *fixed, int32_t *row_ptr, int32_t *col,
+                                           int32_t *val, int32_t *h_out, int64_t *offset_out, int32_t *old_of_new,
+                                           int32_t *n_out, int32_t *scratch)
 {
     __shared__ int s_warp[32];
     __shared__ CsrTotals s_tot;
-    const cg::cluster_group cluster = cg::this_cluster();
-    const int tid = threadIdx.x, rank = blockIdx.x;
-    const int n = S->n, len = (n + kCsrCluster - 1) / kCsrCluster;
+    auto sync = [] {
+        if (NB > 1) cg::this_cluster().sync();
+        else __syncthreads();
+    };
+    const int tid = threadIdx.x, rank = NB > 1 ? blockIdx.x : 0;
+    const int n = S->n, len = (n + NB - 1) / NB;
     const int first = rank * len, last = min(n, first + len);
     const int32_t *srow = S->row_ptr, *scol = S->col, *sval = S->val;
     if (tid == 0) s_tot.off = 0ull;
@@ -131,12 +140,12 @@ __global__ void __cluster_dims__(kCsrCluster, 1, 1) __launch_bounds__(kBigBlock)
         s_tot.nfree = nfree;
         s_tot.nnz = nnz;
     }
-    cluster.sync();  // every block's totals
+    sync();  // every block's totals
 
     int base_n = 0, base_z = 0, m = 0, z = 0;
     unsigned long long osum = 0ull;
-    for (int r = 0; r < kCsrCluster; ++r) {
-        const CsrTotals *t = cluster.map_shared_rank(&s_tot, r);
+    for (int r = 0; r < NB; ++r) {
+        const CsrTotals *t = NB > 1 ? cg::this_cluster().map_shared_rank(&s_tot, r) : &s_tot;
         if (r < rank) {
             base_n += t->nfree;
             base_z += t->nnz;
@@ -162,7 +171,7 @@ __global__ void __cluster_dims__(kCsrCluster, 1, 1) __launch_bounds__(kBigBlock)
             row_ptr[a[u]] = q[u];
         }
     }
-    cluster.sync();  // the new indices, and no block leaves while its totals are read
+    sync();  // the new indices, and no block leaves while its totals are read
 
 #pragma unroll
     for (int u = 0; u < kCsrSpins; ++u) {
@@ -189,6 +198,20 @@ __global__ void __cluster_dims__(kCsrCluster, 1, 1) __launch_bounds__(kBigBlock)
     }
 }
 
+__global__ void __cluster_dims__(kCsrCluster, 1, 1) __launch_bounds__(kBigBlock)
+    k_reduce_csr(const DevProb *S, const int8_t *fixed, int32_t *row_ptr, int32_t *col, int32_t *val,
+                 int32_t *h_out, int64_t *offset_out, int32_t *old_of_new, int32_t *n_out, int32_t *scratch)
+{
+    reduce_csr<kCsrCluster>(S, fixed, row_ptr, col, val, h_out, offset_out, old_of_new, n_out, scratch);
+}
+
+__global__ void __launch_bounds__(kBigBlock)
+    k_reduce_csr_block(const DevProb *S, const int8_t *fixed, int32_t *row_ptr, int32_t *col, int32_t *val,
+                       int32_t *h_out, int64_t *offset_out, int32_t *old_of_new, int32_t *n_out, int32_t *scratch)
+{
+    reduce_csr<1>(S, fixed, row_ptr, col, val, h_out, offset_out, old_of_new, n_out, scratch);
+}
+
 }  // namespace
 }  // namespace spvar
 
@@ -213,7 +236,9 @@ extern "C" int spvar_reduce_noalloc(const spvar_problem *p, const int8_t *fixed,
     const DevProb *src = S->dev;
     void *args[] = {(void *)&src, (void *)&fixed, (void *)&row_ptr, (void *)&col, (void *)&val, (void *)&h,
                     (void *)&offset, (void *)&old_of_new, (void *)&n_out, (void *)&scratch};
-    const cudaError_t e = cudaLaunchKernel(reinterpret_cast<const void *>(k_reduce_csr), dim3(kCsrCluster),
-                                           dim3(kBigBlock), args, 0, reinterpret_cast<cudaStream_t>(stream));
+    const bool one = H.n <= kCsrOneBlock;
+    const cudaError_t e = cudaLaunchKernel(reinterpret_cast<const void *>(one ? k_reduce_csr_block : k_reduce_csr),
+                                           dim3(one ? 1 : kCsrCluster), dim3(kBigBlock), args, 0,
+                                           reinterpret_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? SPVAR_OK : SPVAR_ECUDA;
 }

@@ -29,7 +29,7 @@ def _ring(n, seed):
 
 
 @pytest.mark.parametrize("free", [0.0, 0.15, 0.8])
-@pytest.mark.parametrize("n", [1, 2, 7, 9, 1025, 8191, 8192, 8193, 16384])
+@pytest.mark.parametrize("n", [1, 2, 7, 9, 1025, 2048, 2049, 8191, 8192, 8193, 16384])
 def test_reduce_noalloc_equals_oracle_at_block_edges(cuda_lib, n, free):
     import torch
     spvar = cuda_lib
