@@ -407,11 +407,19 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
                 out.push_back(sh);
         }
     }
-    // few quads: the streaming kernel too (3D L = 9, one start of 69 samples, 114 sweeps: 0.67 ms
-    // against 0.94 for the quad-group kernel)
-    if (quads_ok && pl->C.nslots * ceil_div(pl->C.Smax, 4) <= 2 * pl->sms) {
+    // few quads a launch: the streaming kernel too, and one quad per item (3D L = 9, one start of 69
+    // samples, 114 sweeps: 0.67 ms against 0.94 for the quad-group kernel with more; L = 12, one
+    // launch per start of 250 samples: 24.4 against 50)
+    const int launched = pl->prm.form == SPVAR_FORM_PLAIN ? 1 : pl->C.nslots;
+    if (quads_ok && launched * ceil_div(pl->C.Smax, 4) <= 4 * pl->sms) {
         const int md = pl->max_deg <= 6 ? 6 : 8;
-        for (int b : {256, 512, 1024}) {
+        for (int b : {512, 1024}) {
+            SweepShape sh{6, b, 1, 0, 0, md};
+            if (pm1q_shape_ok(b, md, pl->max_n0, 1) &&
+                sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
+                out.push_back(sh);
+        }
+        for (int b : {128, 256, 512, 1024}) {
             SweepShape sh{2, b, 1, 0, 0, md};
             if (pm1s_shape_ok(b, md, pl->max_n0, 1) &&
                 sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
