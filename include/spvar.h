@@ -374,7 +374,9 @@ typedef struct spvar_params {
                                  n <= 2048 and its 2Rn + 4R(dmax + 1) + 32n bytes in one CTA's
                                  shared memory (else SPVAR_ELIMIT).  Not taken by the server */
 
-#define SPVAR_SWEEP_AUTO 0    /* register kernel when eligible, else general */
+#define SPVAR_SWEEP_AUTO 0    /* plans: the fastest by trial (with a block or replica count given: the
+                                 register kernel when eligible, else general); servers: the quad-group
+                                 kernel for integer couplers where it applies, else general */
 #define SPVAR_SWEEP_GENERAL 1 /* general integer-coupler kernel */
 #define SPVAR_SWEEP_PM1 2     /* register-resident kernel (degree <= 8; |J| = 1 and dmax <= 30 in byte lanes, or
                                  one coupler magnitude per spin, or every |J| <= 15, with dmax <= 4094 in
@@ -383,7 +385,7 @@ typedef struct spvar_params {
 #define SPVAR_SWEEP_PM1W 4    /* warp-per-quad +-1 kernel: replicas_per_block / 4 warps, one quad each */
 #define SPVAR_SWEEP_PM1Q 5    /* quad-group +-1 kernel (|J| = 1, degree <= 8, dmax <= 30): work items of
                                  replicas_per_block / 4 quads of the largest problem (more quads of smaller
-                                 ones, at most 64), spin words alone in shared memory */
+                                 ones, at most 64), two quads per spin word in shared memory */
 /* With the SQA sampler (replicas_per_block = 4): AUTO and PM1 take the register
  * form for +-1 couplers when it applies (two or more slices, at most 4 colour
  * classes, none larger than sweep_block; blocks 256/512/1024), else the item
@@ -476,8 +478,9 @@ typedef struct spvar_server spvar_server;
 
 typedef struct spvar_server_config {
     spvar_params params;    /* Alg. 2 parameters of every request; sweep_kernel = SPVAR_SWEEP_PM1
-                               restricts the server to +-1 couplers (faster sweep: the streaming
-                               +-1 kernel; SPVAR_SWEEP_PM1Q: the quad-group kernel) */
+                               restricts the server to +-1 couplers (the quad-group kernel, or with a
+                               block or replica count given the streaming one; SPVAR_SWEEP_PM1Q: the
+                               quad-group kernel) */
     size_t budget_bytes;    /* device memory for admitted requests' workspaces */
     int32_t max_n;          /* largest request: spins, CSR entries, degree */
     int32_t max_nnz;
@@ -551,7 +554,8 @@ int spvar_plan_post_time(const spvar_plan *plan, double *total_ms);
  * warp-per-quad +-1 kernel, 5: simulated quantum annealing kernel walking
  * (spin, slice) items, 6: simulated quantum annealing kernel in register form:
  * each thread keeps one spin of every colour class in registers and sweeps a
- * fixed set of its slices, 7: quad-group +-1 kernel), persistent grid size. */
+ * fixed set of its slices, 7: quad-group +-1 kernel, 8: quad-group kernel for
+ * integer couplers), persistent grid size. */
 int spvar_plan_shape(const spvar_plan *plan, int32_t *block, int32_t *replicas_per_block,
                      int32_t *staged, int32_t *grid);
 

@@ -8,7 +8,8 @@
 // into bit-sliced counters; fold/compact writes the new CSR, the inherited
 // colour classes and the sweep layout of the smaller problem.  In the
 // multi-start driver one thread-block cluster per start runs all of it in one
-// launch; the standalone entry points and the tree step use one CTA per call.
+// launch, the standalone reduction runs its fold stages on one cluster, and the
+// standalone elite and the tree step use one CTA per call.
 #include <algorithm>
 #include <climits>
 
@@ -617,7 +618,7 @@ static_assert(SPVAR_MAX_N <= 32768, "new index and position are packed in 16 bit
 __device__ __forceinline__ void pass_barrier() { cg::this_cluster().sync(); }
 
 // New index | position << 16 of every old spin (~0 if fixed), in the slot's
-// scratch area (the one-CTA reduction keeps its new indices there).
+// scratch area (the tree step's one-CTA reduction keeps its new indices there).
 __device__ __forceinline__ uint32_t *npos_of(const Slot &s) { return reinterpret_cast<uint32_t *>(s.scratch); }
 
 // Chunks ch[0..G) of the CTA (-1: none) at once, so that the loads of all of
@@ -994,7 +995,8 @@ __device__ __forceinline__ void fold_cluster(Slot &s, int n, int rank)
 
 // The standalone reduction: the pass's fold stages on one cluster.  Bound by
 // the latency of its dependent gathers, which one CTA of 1024 threads walked
-// through a spin at a time.
+// through a spin at a time: 64 us of device time at 8000 spins, about 20 here
+// (the call 150.8 -> 78.7 us, with one allocation and one wait less).
 __global__ void __cluster_dims__(kPassCluster, 1, 1) __launch_bounds__(kPassBlock)
     k_reduce_single(const DevProb *src, DevProb *dst, DevProb hdr, const int8_t *fixed,
                     int32_t *old_of_new, int32_t *scratch)

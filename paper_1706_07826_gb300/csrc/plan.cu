@@ -498,9 +498,11 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
     return out;
 }
 
-// Times a short run of the plan's phases (at most 4, at most 512 sweeps each;
-// the best of two repetitions after an untimed one, and one discarded trial
-// before the first candidate) for every candidate shape and keeps the fastest;
+// Times a short run of the plan's phases (at most 4, 128 sweeps each that step
+// through the whole schedule, up to 512 where a trial is shorter than a
+// millisecond; the best of two repetitions after an untimed one, and one
+// discarded trial before the first candidate) for every candidate shape, the
+// best four once more, and keeps the fastest;
 // results are cached per problem/plan geometry.
 void autotune(spvar_plan *pl, cudaStream_t st, int optin)
 {

@@ -29,7 +29,7 @@
 //
 // Bound: the integer pipes (two 512-thread CTAs an SM, issue active 70 %).  3D L = 10,
 // 304 runs x 32 temperatures, 500 sweeps: 92.5 ms with a byte per spin, byte-wise fields and
-// a queue search per temperature, 30.1 ms now (3.2e11 Metropolis attempts/s).  Of a
+// a queue search per temperature, 28.9 ms now (3.4e11 Metropolis attempts/s).  Of a
 // sweep's time the Metropolis part takes 25 us (150 instructions per four attempts of 32
 // lanes, Philox 70 of them), the cluster moves 20 us (82 us with the queue search: 500
 // instructions a step), the exchanges 4 us and the kept lists 7 us.
