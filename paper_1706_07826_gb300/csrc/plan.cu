@@ -500,10 +500,10 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
 
 // Times a short run of the plan's phases (at most 4, 128 sweeps each that step
 // through the whole schedule, up to 512 where a trial is shorter than a
-// millisecond; the best of two repetitions after an untimed one, and one
-// discarded trial before the first candidate) for every candidate shape, the
-// best four once more, and keeps the fastest;
-// results are cached per problem/plan geometry.
+// millisecond, and four times as many of up to ten phases for the last choice;
+// the best of two repetitions after an untimed one, and one discarded trial
+// before the first candidate) for every candidate shape, the best four once
+// more, and keeps the fastest; results are cached per problem/plan geometry.
 void autotune(spvar_plan *pl, cudaStream_t st, int optin)
 {
     const TuneKey key{pl->max_n0, pl->max_deg, pl->pm1 ? 1 : 0, pl->C.S_fix, pl->C.nslots,
@@ -528,6 +528,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
         pl->trial_rows = std::max(1, pl->T / std::max(Tt, 1));
     };
     set_sweeps(pl->sqa_P > 0 ? 64 : 128);
+    int phases = 4;  // of a trial, at most
     float best = 1e30f;
     SweepShape pick{0, 256, 1, 0, 0, 0};
     bool found = false;
@@ -554,7 +555,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
         C.nslots = nslots;
         const int items = nslots * ceil_div(ceil_div(pl->C.Smax, 4), sh.Q);
         const int grid = (pl->prm.form == SPVAR_FORM_PLAIN) ? items : grid_for(pl, items);
-        const int launches = std::min(pl->iters_max, 4) * launches_per_phase(Tt, chunk_t);
+        const int launches = std::min(pl->iters_max, phases) * launches_per_phase(Tt, chunk_t);
         float ms = 1e30f;
         bool ok = true;
         for (int rep = 0; rep < 3 && ok; ++rep) {
@@ -584,11 +585,18 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
         const float ms = trial(cands[i], 0);
         if (ms < 1e30f) times.emplace_back(ms, i);
     }
-    // the candidates within 5 % of the best, at most four, once more: single trials of nearly
-    // equal shapes pick one that is up to 4 % slower
+    // the candidates within 5 % of the best, at most four, once more, and where that takes a few
+    // milliseconds at four times the sweeps, whose reductions are nearer to the run's: single short
+    // trials of nearly equal shapes pick one that is up to 6 % slower
     std::sort(times.begin(), times.end());
+    const bool longer = !times.empty() && times[0].first < 8.0f && pl->T > Tt;
+    if (longer) {
+        set_sweeps(4 * Tt);
+        phases = 10;
+    }
     for (size_t k = 0; k < times.size() && k < 4 && times[k].first <= 1.05f * times[0].first; ++k) {
-        const float ms = std::min(times[k].first, trial(cands[times[k].second], 0));
+        const float again = trial(cands[times[k].second], 0);
+        const float ms = longer ? again : std::min(times[k].first, again);
         if (ms < best) {
             best = ms;
             pick = cands[times[k].second];

@@ -300,9 +300,11 @@ __device__ void run_item_pm1(const SweepLaunch &L, const SweepJob &job, int quad
     SlotRegs<MAXD> s[NSLOT];
     uint32_t barmask = 0;
     RoundKeys K;
-    // small integer couplers: 2.7 % faster with the keys formed behind the slots (U_10 Chimera C8, 2000
-    // samples, 1000 sweeps: 1538 -> 1497 us); the byte-lane forms up to 14 % slower
-    if (!SI) K = philox_keys<3>(k0, k1);
+    // small integer couplers in four slots: 2.7 % faster with the keys formed behind the slots (U_10
+    // Chimera C8, 2000 samples, 1000 sweeps: 1538 -> 1497 us); in two slots up to 2 %, the byte-lane
+    // forms up to 14 % slower
+    constexpr bool kKeysLate = SI && NSLOT > 2;
+    if (!kKeysLate) K = philox_keys<3>(k0, k1);
     const uint32_t dummy = 4u * (uint32_t)(KW - 1), zero = 4u * (uint32_t)(2 * KW);
 #pragma unroll
     for (int j = 0; j < NSLOT; ++j) {
@@ -361,7 +363,7 @@ __device__ void run_item_pm1(const SweepLaunch &L, const SweepJob &job, int quad
             }
         }
     }
-    if (SI) K = philox_keys<3>(k0, k1);
+    if (kKeysLate) K = philox_keys<3>(k0, k1);
     const uint32_t k16 = SCALED ? (uint32_t)(32 * bias) * 0x00010001u : (uint32_t)(16 * bias) * 0x01010101u;
     const uint32_t *thr = L.thr;
     const size_t ts = (size_t)L.thr_stride;
