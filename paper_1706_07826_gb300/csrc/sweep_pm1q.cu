@@ -418,8 +418,10 @@ __device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int qua
         }
     for (int x = tid; x < np * ns; x += B) {
         const int v = x / ns, p = x - v * ns;
+        // quads past the item's end start at 0: a resumed sample reads the rows another block may be writing,
+        // and only an item's own rows are safe to read
         uint32_t w = 0u;
-        if (p < n) {
+        if (p < n && 2 * v < nq) {
             w = start_word(P, job, quad0 + 2 * v, p);
             if (2 * v + 1 < nq) w |= start_word(P, job, quad0 + 2 * v + 1, p) << 4;
         }
