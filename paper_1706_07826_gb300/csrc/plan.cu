@@ -39,7 +39,7 @@ cudaError_t engine_phase(const PhaseEngine &E, Slot *slots, int nslots, int T, i
     C.Q = E.shape.Q;
     C.fit_block = E.shape.kind == 1 ? E.shape.block : 0;
     C.fit_nslot = E.shape.kind == 1 ? E.shape.nslot : 0;
-    QuadLayout ql{1, 0, 0, 0, 0};
+    QuadLayout ql{1, 0, 0, 0, 0, false, 0};
     if (E.shape.kind == 6) ql = pm1q_layout(E.shape.block, E.max_n0, E.shape.Q, E.shape.maxd);
     if (E.shape.kind == 7) {
         const GqLayout gl = gq_layout(E.shape.block, E.max_n0, E.shape.Q, E.shape.maxd, E.thr_stride, kSmemOptin);
@@ -402,9 +402,7 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
         const int shapes[][2] = {{128, 2}, {128, 4}, {256, 2}, {256, 4}, {256, 8}, {512, 2}, {512, 4}, {512, 8}, {1024, 2}, {1024, 16}};
         for (const auto &bq : shapes) {
             SweepShape sh{6, bq[0], bq[1], 0, 0, md};
-            if (pm1q_shape_ok(bq[0], md, pl->max_n0, bq[1]) &&
-                sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
-                out.push_back(sh);
+            if (pm1q_fits(bq[0], pl->max_n0, bq[1], md, (size_t)optin)) out.push_back(sh);
         }
     }
     // few quads a launch: the streaming kernel too, and one quad per item (3D L = 9, one start of 69
@@ -415,9 +413,7 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
         const int md = pl->max_deg <= 6 ? 6 : 8;
         for (int b : {512, 1024}) {
             SweepShape sh{6, b, 1, 0, 0, md};
-            if (pm1q_shape_ok(b, md, pl->max_n0, 1) &&
-                sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
-                out.push_back(sh);
+            if (pm1q_fits(b, pl->max_n0, 1, md, (size_t)optin)) out.push_back(sh);
         }
         for (int b : {128, 256, 512, 1024}) {
             SweepShape sh{2, b, 1, 0, 0, md};
@@ -946,8 +942,8 @@ int spvar_plan_create(const spvar_problem *const *problems, int32_t nproblems,
             }
         } else if (p.sweep_kernel == SPVAR_SWEEP_PM1Q) {
             const int md = pl->max_deg <= 6 ? 6 : 8;
-            if (!pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg) || !pm1q_shape_ok(blk, md, pl->max_n0, Q) ||
-                !pm1q_request_ok(pl->max_n0, Q, (size_t)optin)) {
+            if (!pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg) ||
+                !pm1q_request_ok(blk, pl->max_n0, Q, md, (size_t)optin)) {
                 plan_free(pl);
                 return SPVAR_ELIMIT;
             }

@@ -516,7 +516,7 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
     if (pm1_only && want_quads && cfg->max_degree <= 8 && cfg->max_dmax <= 30) {
         const int qb = (p.sweep_block == 128 || p.sweep_block == 256) ? p.sweep_block : 512;
         SweepShape sh{6, qb, Q, 0, 0, md};
-        if (pm1q_shape_ok(qb, md, cfg->max_n, Q) && pm1q_request_ok(cfg->max_n, Q, (size_t)optin)) {
+        if (pm1q_request_ok(qb, cfg->max_n, Q, md, (size_t)optin)) {
             E.shape = sh;
             chosen = true;
         }

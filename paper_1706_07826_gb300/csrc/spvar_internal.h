@@ -393,11 +393,18 @@ struct QuadLayout {
     int nv, rec, unit_rows;  // pairs of quads per group, words of a spin's record (0: none), listed rounds of units
     int fit_words;           // words for records and groups
     size_t bytes;            // dynamic shared memory
+    bool tabs;               // the kernel with the second acceptance table
+    size_t stat;             // its static shared memory
 };
 QuadLayout pm1q_layout(int block, int max_n, int Q, int maxd);
 SweepShape pm1q_default(int max_n, int maxd, size_t optin);
-// A requested item of Q quads is taken where two copies of every quad's spin words fit a CTA.
-inline bool pm1q_request_ok(int max_n, int Q, size_t optin) { return 8 * (size_t)Q * ((size_t)max_n + 1) <= optin; }
+// The kernel exists and its static and dynamic shared memory fit a CTA.
+bool pm1q_fits(int block, int max_n, int Q, int maxd, size_t optin);
+// A requested item of Q quads is taken where two copies of every quad's spin words, and the launch itself, fit a CTA.
+inline bool pm1q_request_ok(int block, int max_n, int Q, int maxd, size_t optin)
+{
+    return 8 * (size_t)Q * ((size_t)max_n + 1) <= optin && pm1q_fits(block, max_n, Q, maxd, optin);
+}
 cudaError_t launch_sweep_pm1q(const SweepLaunch &L, int block, int maxd, int Q, int grid, size_t smem, cudaStream_t st);
 int pm1q_max_active_blocks(int block, int maxd, int max_n, int Q, size_t smem);
 

@@ -33,8 +33,8 @@ namespace {
 
 constexpr int kQcap = 64;           // most quads per work item
 constexpr int kPcap = kQcap / 2;    // most pairs
-constexpr size_t kQuadStatic = 7 << 10;     // static shared memory and the system's 1 KB, rounded up
-constexpr size_t kQuadSmemMax = 218 << 10;  // dynamic shared memory records may bring a CTA to (the static part is 6 KB)
+constexpr size_t kQuadRoom = 7 << 10;       // left beside a CTA's dynamic part where a default shape is chosen
+constexpr size_t kQuadSmemMax = 218 << 10;  // dynamic shared memory records may bring a CTA to
 constexpr uint32_t kM = 0x01010101u, kN = 0x11111111u, kOdd = 0x10101010u;
 
 // NV words (one of every pair of a group) at once.
@@ -65,7 +65,8 @@ __device__ __forceinline__ void sts_nv(uint32_t a, const uint32_t (&v)[NV])
 // (c8 / 4) * 64 + 4 z + c8 % 4, so a nibble of z in the high half of a byte is already
 // the entry's byte offset in its 256-byte block.  One comparison accepts; the table
 // cannot hold thr = 0 (never accept), so sweeps whose row has one (large beta) use the
-// first form.
+// first form.  So do launches without the table: degree 7 and 8, and a lone pair of a
+// problem whose spin words leave no room for its 4 KB.
 constexpr int kTabWords = 8 * 64;
 
 // Acceptance rows of the current and the next sweep: the threshold of flip cost
@@ -74,14 +75,20 @@ constexpr int kTabWords = 8 * 64;
 // that is ignored).  Costs |e| <= 7, all a +-1 problem without large biases has, lie
 // on different banks.  Rows are 256-byte aligned: the index byte replaces the low byte
 // of the row's address.
+template <bool TABS>
 struct QuadSmem {
     uint32_t row[2][64];
-    uint32_t tab[2][kTabWords];  // see below
+    uint32_t tab[TABS ? 2 : 1][TABS ? kTabWords : 4];
     int zero[2];                 // the row holds a threshold of 0
     int c8lo, c8hi;              // range of the problem's flip-cost constants
     int e2[4 * kQcap];
     int4 cls[kMaxColours];  // per colour class, as unit_classes fills it
+    int item;               // the queue's next work item
 };
+constexpr size_t quad_static(bool tabs) { return tabs ? sizeof(QuadSmem<true>) : sizeof(QuadSmem<false>); }
+// a CTA takes 1 KB of the system's beside its own; an SM has 1 KB more than one CTA may take
+static_assert(2 * (quad_static(true) + 1024) <= 2 * kQuadRoom + 1024, "two CTAs of a default shape share an SM");
+static_assert(kQuadSmemMax + quad_static(true) <= kSmemOptin, "records and the static part fit a CTA");
 
 // One quad's four acceptance tests: adds 1 << (8r + SH) to rej for every replica r whose
 // word is not below its threshold.
@@ -186,8 +193,8 @@ struct QuadItem {
 // One sweep, on acceptance row PAR (the sweep's parity: its row is at a compile-time
 // address); y1 is the next sweep's counter word and next_thr its threshold row (null
 // after the last sweep).
-template <int B, int MAXD, int NV, bool STAGED, int PAR, bool TAB>
-__device__ __forceinline__ void sweep_pairs(const QuadItem &I, QuadSmem &sm, uint32_t *pairs, const uint4 *rec,
+template <int B, int MAXD, int NV, bool STAGED, int PAR, bool TAB, bool TABS>
+__device__ __forceinline__ void sweep_pairs(const QuadItem &I, QuadSmem<TABS> &sm, uint32_t *pairs, const uint4 *rec,
                                             const uint32_t *rec2, const uint32_t *unit, uint32_t y1,
                                             const uint32_t *__restrict__ next_thr, const PhiloxKeys<2> &K)
 {
@@ -203,7 +210,7 @@ __device__ __forceinline__ void sweep_pairs(const QuadItem &I, QuadSmem &sm, uin
             if (tid == 0) sm.zero[PAR ^ 1] = zero;
         }
         // loaded here, stored after the first class
-        if (MAXD == 6 && tid < tabs) top = top_word(next_thr, sm.c8lo + (tid >> 4), tid & 15, I.bias);
+        if (TABS && tid < tabs) top = top_word(next_thr, sm.c8lo + (tid >> 4), tid & 15, I.bias);
         if (tid < I.np) {
             uint4 *head = reinterpret_cast<uint4 *>(pairs + (size_t)(tid / NV) * (I.v4 / 4)) + tid % NV;
             const uint4 h = head[2 * NV];
@@ -213,7 +220,7 @@ __device__ __forceinline__ void sweep_pairs(const QuadItem &I, QuadSmem &sm, uin
             head[(PAR ^ 1) * NV] = q;
         }
     }
-    const uint32_t row = shared_addr(TAB ? sm.tab[PAR] : sm.row[PAR]);
+    const uint32_t row = shared_addr(TAB ? sm.tab[TABS ? PAR : 0] : sm.row[PAR]);
     const uint32_t first = I.sw4, last = I.sw4 + I.end4;
     for (int c = 0; c < I.ncol; ++c) {
         const int4 cl = sm.cls[c];
@@ -329,30 +336,32 @@ __device__ __forceinline__ void sweep_pairs(const QuadItem &I, QuadSmem &sm, uin
                 } while (base < last);
             }
         }
-        if (MAXD == 6 && c == 0 && next_thr) {
-            if (tid < tabs) sm.tab[PAR ^ 1][tab_word(sm.c8lo + (tid >> 4), tid & 15)] = top;
-            for (int i = tid + B; i < tabs; i += B)
-                sm.tab[PAR ^ 1][tab_word(sm.c8lo + (i >> 4), i & 15)] =
-                    top_word(next_thr, sm.c8lo + (i >> 4), i & 15, I.bias);
+        if constexpr (TABS) {
+            if (c == 0 && next_thr) {
+                if (tid < tabs) sm.tab[PAR ^ 1][tab_word(sm.c8lo + (tid >> 4), tid & 15)] = top;
+                for (int i = tid + B; i < tabs; i += B)
+                    sm.tab[PAR ^ 1][tab_word(sm.c8lo + (i >> 4), i & 15)] =
+                        top_word(next_thr, sm.c8lo + (i >> 4), i & 15, I.bias);
+            }
         }
         __syncthreads();
     }
 }
 
 // The form the sweep's acceptance row allows.
-template <int B, int MAXD, int NV, bool STAGED, int PAR>
-__device__ __forceinline__ void sweep_pairs_par(const QuadItem &I, QuadSmem &sm, uint32_t *pairs, const uint4 *rec,
+template <int B, int MAXD, int NV, bool STAGED, int PAR, bool TABS>
+__device__ __forceinline__ void sweep_pairs_par(const QuadItem &I, QuadSmem<TABS> &sm, uint32_t *pairs, const uint4 *rec,
                                                 const uint32_t *rec2, const uint32_t *unit, uint32_t y1,
                                                 const uint32_t *next_thr, const PhiloxKeys<2> &K)
 {
-    if (MAXD == 6 && !sm.zero[PAR])
-        sweep_pairs<B, MAXD, NV, STAGED, PAR, true>(I, sm, pairs, rec, rec2, unit, y1, next_thr, K);
+    if (TABS && !sm.zero[PAR])
+        sweep_pairs<B, MAXD, NV, STAGED, PAR, TABS>(I, sm, pairs, rec, rec2, unit, y1, next_thr, K);
     else
         sweep_pairs<B, MAXD, NV, STAGED, PAR, false>(I, sm, pairs, rec, rec2, unit, y1, next_thr, K);
 }
 
-template <int B, int MAXD, int NV, bool STAGED>
-__device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int quad0, int nq, QuadSmem &sm,
+template <int B, int MAXD, int NV, bool STAGED, bool TABS>
+__device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int quad0, int nq, QuadSmem<TABS> &sm,
                               uint32_t *smem)
 {
     const int tid = threadIdx.x;
@@ -453,7 +462,7 @@ __device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int qua
             sm.row[t0 & 1][2 * (tid + 1) + 30] = v;
             if (v == 0u) sm.zero[t0 & 1] = 1;
         }
-        if (MAXD == 6)
+        if constexpr (TABS)
             for (int i = tid; i < 16 * (sm.c8hi - sm.c8lo + 1); i += B)
                 sm.tab[t0 & 1][tab_word(sm.c8lo + (i >> 4), i & 15)] = top_word(row, sm.c8lo + (i >> 4), i & 15, bias);
     }
@@ -494,31 +503,33 @@ __device__ void run_item_pm1q(const SweepLaunch &L, const SweepJob &job, int qua
     finish_pairs<NV>(P, job, quad0, nq, sw, sm.e2);
 }
 
-template <int B, int MAXD, int NV, bool STAGED>
+template <int B, int MAXD, int NV, bool STAGED, bool TABS>
 __global__ void __launch_bounds__(B, 1024 / B) k_sweep_pm1q(const SweepLaunch L)
 {
-    __shared__ __align__(256) QuadSmem sm;
+    __shared__ __align__(256) QuadSmem<TABS> sm;
     extern __shared__ __align__(16) uint32_t smem_pm1q[];
-    __shared__ int s_item;
     for (int iter = 0;; ++iter) {
         SweepJob job;
         int quad0, nq;
-        if (!next_item(L, iter, &s_item, job, quad0, nq)) break;
-        run_item_pm1q<B, MAXD, NV, STAGED>(L, job, quad0, nq, sm, smem_pm1q);
+        if (!next_item(L, iter, &sm.item, job, quad0, nq)) break;
+        run_item_pm1q<B, MAXD, NV, STAGED, TABS>(L, job, quad0, nq, sm, smem_pm1q);
         __syncthreads();
     }
 }
 
-void *select_q(int block, int maxd, int nv, bool staged)
+void *select_q(int block, int maxd, int nv, bool staged, bool tabs)
 {
-#define SPVAR_PM1Q_CASE(BB, MD, NVV)                                                         \
-    if (block == BB && maxd == MD && nv == NVV)                                              \
-        return staged ? reinterpret_cast<void *>(k_sweep_pm1q<BB, MD, NVV, true>)            \
-                      : reinterpret_cast<void *>(k_sweep_pm1q<BB, MD, NVV, false>);
-#define SPVAR_PM1Q_NV(BB, MD) SPVAR_PM1Q_CASE(BB, MD, 1) SPVAR_PM1Q_CASE(BB, MD, 2)
-    SPVAR_PM1Q_NV(128, 6) SPVAR_PM1Q_NV(256, 6) SPVAR_PM1Q_NV(512, 6) SPVAR_PM1Q_NV(1024, 6)
-    SPVAR_PM1Q_NV(128, 8) SPVAR_PM1Q_NV(256, 8) SPVAR_PM1Q_NV(512, 8) SPVAR_PM1Q_NV(1024, 8)
-#undef SPVAR_PM1Q_NV
+#define SPVAR_PM1Q_CASE(BB, MD, NVV, ST, TB)                              \
+    if (block == BB && maxd == MD && nv == NVV && staged == ST && tabs == TB) \
+        return reinterpret_cast<void *>(k_sweep_pm1q<BB, MD, NVV, ST, TB>);
+#define SPVAR_PM1Q_BLOCK(BB)                                                                              \
+    SPVAR_PM1Q_CASE(BB, 6, 1, true, true) SPVAR_PM1Q_CASE(BB, 6, 2, true, true)                           \
+    SPVAR_PM1Q_CASE(BB, 6, 1, false, true) SPVAR_PM1Q_CASE(BB, 6, 2, false, true)                         \
+    SPVAR_PM1Q_CASE(BB, 6, 1, false, false)                                                               \
+    SPVAR_PM1Q_CASE(BB, 8, 1, true, false) SPVAR_PM1Q_CASE(BB, 8, 2, true, false)                         \
+    SPVAR_PM1Q_CASE(BB, 8, 1, false, false) SPVAR_PM1Q_CASE(BB, 8, 2, false, false)
+    SPVAR_PM1Q_BLOCK(128) SPVAR_PM1Q_BLOCK(256) SPVAR_PM1Q_BLOCK(512) SPVAR_PM1Q_BLOCK(1024)
+#undef SPVAR_PM1Q_BLOCK
 #undef SPVAR_PM1Q_CASE
     return nullptr;
 }
@@ -528,7 +539,7 @@ void *select_q(int block, int maxd, int nv, bool staged)
 // Q quads of a problem of at most max_n spins per work item.
 bool pm1q_shape_ok(int block, int maxd, int max_n, int Q)
 {
-    return select_q(block, maxd, 1, false) != nullptr && Q >= 1 && Q <= kQcap && max_n < 0xFFFF;
+    return select_q(block, maxd, 1, false, false) != nullptr && Q >= 1 && Q <= kQcap && max_n < 0xFFFF;
 }
 
 // Pairs of quads per group (one vector load).
@@ -558,7 +569,17 @@ QuadLayout pm1q_layout(int block, int max_n, int Q, int maxd)
     }
     l.fit_words = (int)((l.rec ? recs : 0) + groups);
     l.bytes = 4 * ((size_t)l.fit_words + (size_t)l.unit_rows * block);
+    // the second table everywhere but in a lone pair's last 4 KB (28276 .. 28787 spins), the one place where a
+    // problem that ran without it would not fit a CTA with it
+    l.tabs = maxd <= 6 && (l.rec > 0 || l.nv > 1 || l.bytes + quad_static(true) <= kSmemOptin);
+    l.stat = quad_static(l.tabs);
     return l;
+}
+
+bool pm1q_fits(int block, int max_n, int Q, int maxd, size_t optin)
+{
+    const QuadLayout l = pm1q_layout(block, max_n, Q, maxd);
+    return pm1q_shape_ok(block, maxd, max_n, Q) && l.bytes + l.stat <= optin;
 }
 
 // Block and quads per item for problems of at most max_n spins where nothing is tuned:
@@ -570,16 +591,16 @@ QuadLayout pm1q_layout(int block, int max_n, int Q, int maxd)
 SweepShape pm1q_default(int max_n, int maxd, size_t optin)
 {
     for (int Q : {8, 4, 2})
-        if (2 * (pm1q_layout(512, max_n, Q, maxd).bytes + kQuadStatic) <= optin) return SweepShape{6, 512, Q, 0, 0, maxd};
+        if (2 * (pm1q_layout(512, max_n, Q, maxd).bytes + kQuadRoom) <= optin) return SweepShape{6, 512, Q, 0, 0, maxd};
     for (int Q : {2, 1})
-        if (pm1q_layout(1024, max_n, Q, maxd).bytes + kQuadStatic <= optin) return SweepShape{6, 1024, Q, 0, 0, maxd};
+        if (pm1q_layout(1024, max_n, Q, maxd).bytes + kQuadRoom <= optin) return SweepShape{6, 1024, Q, 0, 0, maxd};
     return SweepShape{6, 0, 1, 0, 0, maxd};
 }
 
 cudaError_t launch_sweep_pm1q(const SweepLaunch &L, int block, int maxd, int Q, int grid, size_t smem, cudaStream_t st)
 {
     const QuadLayout l = pm1q_layout(block, L.max_n, Q, maxd);
-    void *k = select_q(block, maxd, l.nv, l.rec > 0);
+    void *k = select_q(block, maxd, l.nv, l.rec > 0, l.tabs);
     if (!k) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -592,7 +613,7 @@ cudaError_t launch_sweep_pm1q(const SweepLaunch &L, int block, int maxd, int Q, 
 int pm1q_max_active_blocks(int block, int maxd, int max_n, int Q, size_t smem)
 {
     const QuadLayout l = pm1q_layout(block, max_n, Q, maxd);
-    void *k = select_q(block, maxd, l.nv, l.rec > 0);
+    void *k = select_q(block, maxd, l.nv, l.rec > 0, l.tabs);
     if (!k) return 0;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int nb = 0;
