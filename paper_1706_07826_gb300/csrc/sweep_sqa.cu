@@ -194,8 +194,18 @@ __device__ __forceinline__ void sqa_reg_pass(uint32_t sw4, uint32_t row, int g, 
     }
 }
 
+// Static shared memory.  The register form's is 256 bytes, so that the dynamic part behind it,
+// which begins with the acceptance rows, starts on a 256-byte boundary; the walk needs no
+// alignment, and a larger static part would take from the problems that fit it.
+template <bool REG>
+struct alignas(REG ? 256 : 16) SqaStatic {
+    int cptr[kMaxColours + 1];
+    int item;  // the queue's next work item
+};
+static_assert(sizeof(SqaStatic<true>) == 256 && sizeof(SqaStatic<false>) == 144, "static parts of both forms");
+
 template <bool PM1, int B, int MAXD, int NC, int E, bool SI>
-__device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad, uint32_t *smem)
+__device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad, int *s_cptr, uint32_t *smem)
 {
     const int tid = threadIdx.x;
     const DevProb *pr = job.prob;
@@ -216,7 +226,6 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
     uint16_t *off = reinterpret_cast<uint16_t *>(idx_s + n);                 // [MAXD][n] (+-1)
     int *e2 = reinterpret_cast<int *>(REG ? meta_s : idx_s + n + (PM1 ? ((size_t)MAXD * n + 1) / 2 : 0));
     int *s_best = e2 + 4 * P;
-    __shared__ int s_cptr[kMaxColours + 1];
 
     for (int c = tid; c <= ncol; c += B) s_cptr[c] = pr->cptr[c];
     if (!REG)
@@ -487,13 +496,13 @@ constexpr int sqa_min_blocks()
 template <bool PM1, int B, int MAXD, int NC, int E, bool SI>
 __global__ void __launch_bounds__(B, sqa_min_blocks<B, MAXD, NC, SI>()) k_sweep_sqa(const SweepLaunch L)
 {
-    extern __shared__ __align__(256) uint32_t smem_sqa[];
-    __shared__ int s_item;
+    extern __shared__ __align__(16) uint32_t smem_sqa[];
+    __shared__ SqaStatic<(NC > 0)> sm;
     for (int iter = 0;; ++iter) {
         SweepJob job;
         int quad0, nq;
-        if (!next_item(L, iter, &s_item, job, quad0, nq)) break;
-        run_item_sqa<PM1, B, MAXD, NC, E, SI>(L, job, quad0, smem_sqa);
+        if (!next_item(L, iter, &sm.item, job, quad0, nq)) break;
+        run_item_sqa<PM1, B, MAXD, NC, E, SI>(L, job, quad0, sm.cptr, smem_sqa);
         __syncthreads();
     }
 }
