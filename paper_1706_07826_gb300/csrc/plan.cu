@@ -98,19 +98,10 @@ cudaError_t engine_phase(const PhaseEngine &E, Slot *slots, int nslots, int T, i
 
 }  // namespace spvar
 
-struct spvar_plan {
+struct spvar_plan : PlanGeometry {
     int device = 0;
-    std::vector<const Problem *> probs;
     std::vector<int> starts_of;  // slot -> problem
-    spvar_params prm{};
-    SolveConsts C{};
     int trial_rows = 1;  // rows of the schedule per sweep (more than one in the autotuner's trials)
-    int T = 0, thr_stride = 1, max_n0 = 0, max_deg = 1, iters_max = 1;
-    int ncol_max = 0, class_max = 0;  // most colour classes and largest class of any problem
-    int jabs_max = 0;                 // largest coupler magnitude of any problem
-    bool pm1 = true;
-    bool ujs = true;      // every problem has one coupler magnitude per spin
-    uint64_t sig = 0;     // structure signature of the problems (autotune cache key)
     void *ws = nullptr;
     size_t ws_bytes = 0;
     Slot *d_slots = nullptr;
@@ -118,12 +109,10 @@ struct spvar_plan {
     Slot *h_slots_pinned = nullptr;
     uint32_t *d_thr = nullptr;
     unsigned long long *d_ent = nullptr;  // SQA acceptance entries
-    int sqa_P = 0, sqa_W = 0;             // SQA slices and table width (0: SA)
     // PTICM as the sampler: temperatures, kept states per list, exchange-table width, tables
     int pt_R = 0, pt_K = 0, pt_dx = 0;
     uint32_t *d_pt_thr = nullptr, *d_pt_xthr = nullptr;
     size_t pt_smem = 0;
-    bool sqa_ent32 = false;               // SQA: no acceptance entry is 2^32 (32-bit entries suffice)
     SweepJob *d_jobs = nullptr;
     WorkItem *d_items = nullptr;
     int32_t *d_ctr = nullptr;       // [0] nitems, [1] queue, [2] nactive, [3] phases run by the loop graph
@@ -134,7 +123,7 @@ struct spvar_plan {
     int8_t *d_fmap = nullptr, *d_best = nullptr;
     size_t fmap_total = 0;
     SweepShape shape{0, 256, 1, 0, 0, 0};
-    int sweep_grid = 1, sms = 1, dmax = 0;
+    int sweep_grid = 1;
     size_t sweep_smem = 0;
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph = nullptr;       // one batched phase
@@ -341,7 +330,7 @@ int upload_slots(spvar_plan *pl, const uint64_t *seeds, cudaStream_t st)
 }
 
 // Register-kernel slot count covering every problem of the plan (0 if none).
-int plan_nslot(const spvar_plan *pl, int Q, int block)
+int plan_nslot(const PlanGeometry *pl, int Q, int block)
 {
     int ns = 2;
     for (const Problem *P : pl->probs) {
@@ -352,11 +341,9 @@ int plan_nslot(const spvar_plan *pl, int Q, int block)
     return ns;
 }
 
-// Candidate sweep shapes for a plan: the general kernel with and without the
-// staged layout, and (for +-1 problems) the register-resident kernel.
 // SQA sweep shape of a variant (0 general, 1 +-1 walk, 2 +-1 register form)
 // and block size, or kind -1 if it does not apply or the slices do not fit.
-SweepShape sqa_shape(const spvar_plan *pl, int block, int optin, int variant)
+SweepShape sqa_shape(const PlanGeometry *pl, int block, int optin, int variant)
 {
     SweepShape sh{5, block, 1, variant, pl->sqa_W, pl->max_deg};
     sh.slices = pl->sqa_P;
@@ -372,7 +359,11 @@ SweepShape sqa_shape(const spvar_plan *pl, int block, int optin, int variant)
     return sh;
 }
 
-std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
+}  // namespace
+
+namespace spvar {
+
+std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin)
 {
     std::vector<SweepShape> out;
     if (pl->sqa_P > 0) {
@@ -390,11 +381,11 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
         }
         return out;
     }
-    // +-1 couplers and dmax <= 30: the quad-group and the register kernel.  The streaming, the
-    // warp-per-quad and the general kernel lost to the quad-group kernel at every size measured
-    // (3D L = 9, 20 starts x (250 + 250): 6.4 ms against 9.3 ms warp per quad and 13.2 ms
-    // streaming; L = 12: 10.8 against 14.0 streaming; the uneven batch of L = 6 .. 12: 37 against
-    // 104), so they are tried only where it does not apply.
+    // Quad-group kernels first, where they apply: for +-1 couplers and dmax <= 30 the streaming, the
+    // warp-per-quad and the general kernel lost to theirs at every size measured with many quads (3D
+    // L = 9, 20 starts x (250 + 250): 6.4 ms against 9.3 ms warp per quad and 13.2 ms streaming; L = 12:
+    // 10.8 against 14.0 streaming; the uneven batch of L = 6 .. 12: 37 against 104), for integer couplers
+    // the general one (see there).  The exceptions follow at each kernel.
     const bool quads_ok = pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg);
     const size_t listed = out.size();
     if (quads_ok) {
@@ -431,8 +422,11 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
             if (gq_layout(bq[0], pl->max_n0, bq[1], md, pl->thr_stride, (size_t)optin).nw > 0)
                 out.push_back(SweepShape{7, bq[0], bq[1], 0, 0, md});
     }
-    const bool others = out.size() == listed;
-    if (others && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
+    const bool others = out.size() == listed;  // no quad-group kernel applies
+    // +-1 couplers with large biases (dmax 31 .. 254): a warp per quad, and the streaming kernel (200 sweeps,
+    // dmax 32: L = 9, 20 starts x (250 + 250) 2.52 ms warp per quad, 3.34 the integer quad groups; L = 4 0.65
+    // and 0.74; L = 14, 8 starts x (200 + 200), four phases 3.99 ms streaming and 4.20)
+    if ((others || !quads_ok) && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
         const int md = pl->max_deg <= 6 ? 6 : 8;
         for (int w : {2, 4, 8, 16})
             for (int K : {2, 4}) {
@@ -441,6 +435,12 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
                     sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
                     out.push_back(sh);
             }
+        for (int b : {128, 256, 512, 1024}) {
+            SweepShape sh{2, b, 1, 0, 0, md};
+            if (pm1s_shape_ok(b, md, pl->max_n0, 1) &&
+                sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
+                out.push_back(sh);
+        }
     }
     const int blocks[3] = {128, 256, 512};
     const int qs[4] = {1, 2, 4, 8};
@@ -452,16 +452,6 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
             for (int stg = 1; others && stg >= 0; --stg) {
                 SweepShape sh{0, blocks[bi], Q, stg, 0, 0};
                 if (sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin) out.push_back(sh);
-            }
-            if (others && Q == 1 && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
-                const int md = pl->max_deg <= 6 ? 6 : 8;
-                for (int sb : {128, 256, 512, 1024}) {
-                    if (sb != blocks[bi] && !(bi == 2 && sb == 1024)) continue;
-                    SweepShape sh{2, sb, 1, 0, 0, md};
-                    if (pm1s_shape_ok(sb, md, pl->max_n0, 1) &&
-                        sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
-                        out.push_back(sh);
-                }
             }
             if (pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
                 const int ns = plan_nslot(pl, Q, blocks[bi]);
@@ -493,6 +483,10 @@ std::vector<SweepShape> candidate_shapes(const spvar_plan *pl, int optin)
     }
     return out;
 }
+
+}  // namespace spvar
+
+namespace {
 
 // Times a short run of the plan's phases (at most 4, 128 sweeps each that step
 // through the whole schedule, up to 512 where a trial is shorter than a

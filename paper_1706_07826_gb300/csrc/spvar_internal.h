@@ -503,6 +503,24 @@ inline int sweep_shape_occupancy(const SweepShape &s, bool pm1, int max_n, int t
     return sweep_max_active_blocks(pm1, s.block, smem, s.stage != 0);
 }
 
+// What the choice of a plan's sweep shape depends on.
+struct PlanGeometry {
+    std::vector<const Problem *> probs;
+    spvar_params prm{};
+    SolveConsts C{};
+    int T = 0, thr_stride = 1, max_n0 = 0, max_deg = 1, iters_max = 1;
+    int ncol_max = 0, class_max = 0;  // most colour classes and largest class of any problem
+    int jabs_max = 0;                 // largest coupler magnitude of any problem
+    int dmax = 0, sms = 1;
+    bool pm1 = true;
+    bool ujs = true;                  // every problem has one coupler magnitude per spin
+    int sqa_P = 0, sqa_W = 0;         // SQA slices and table width (0: SA)
+    bool sqa_ent32 = false;           // SQA: no acceptance entry is 2^32 (32-bit entries suffice)
+    uint64_t sig = 0;                 // structure signature of the problems (autotune cache key)
+};
+// Sweep shapes the autotuner times for a plan.
+std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin);
+
 // Everything one Multi-start SPVAR phase needs besides the slots.
 struct PhaseEngine {
     SweepShape shape;

@@ -24,6 +24,31 @@ int main(int argc, char **argv)
         std::printf("%d %zu %d\n", (int)pm1q_request_ok(arg(2), arg(3), arg(4), arg(5), kSmemOptin), l.bytes + l.stat,
                     (int)l.tabs);
     }
+    if (!std::strcmp(argv[1], "candidates")) {
+        // spins, colour classes (of equal size), degree, dmax, +-1, largest coupler, starts, samples, plain form:
+        // kind and quads per item of every shape the autotuner times
+        Problem P;
+        std::memset(&P.hdr, 0, sizeof(P.hdr));
+        P.hdr.n = arg(2);
+        P.hdr.ncol = arg(3);
+        for (int c = 0; c < arg(3); ++c) P.csize[c] = arg(2) / arg(3) + (c < arg(2) % arg(3));
+        P.jabs_max = arg(7);
+        PlanGeometry g;
+        g.probs.push_back(&P);
+        g.prm.form = arg(10) ? SPVAR_FORM_PLAIN : SPVAR_FORM_BATCHED;
+        g.C.S_fix = g.C.S_solve = g.C.Smax = arg(9);
+        g.C.nslots = arg(8);
+        g.max_n0 = arg(2);
+        g.max_deg = arg(4);
+        g.dmax = arg(5);
+        g.thr_stride = arg(5) + 1;
+        g.jabs_max = arg(7);
+        g.pm1 = g.ujs = arg(6) != 0;
+        g.ncol_max = arg(3);
+        g.class_max = P.csize[0];
+        g.sms = 152;
+        for (const SweepShape &s : candidate_shapes(&g, kSmemOptin)) std::printf("%d:%d:%d ", s.kind, s.block, s.Q);
+    }
     return 0;
 }
 """
@@ -56,3 +81,25 @@ def test_requested_quads_are_taken_where_the_launch_fits(rules, maxd):
         if n < 28200:
             assert int(tabs) == (maxd == 6)
     assert rules("request", 256, 28800, 1, maxd)[0] == "0"
+
+
+GENERAL, REGISTER, STREAMING, WARP, QUADS, INTEGER_QUADS = 0, 1, 2, 4, 6, 7
+
+
+def _kinds(rules, n, deg=6, dmax=12, pm1=True, jmax=1, starts=20, samples=250, plain=False, ncol=2):
+    out = rules("candidates", n, ncol, deg, dmax, int(pm1), jmax, starts, samples, int(plain))
+    return {int(x.split(":")[0]) for x in out}
+
+
+@pytest.mark.parametrize("dmax", [32, 100, 254])
+@pytest.mark.parametrize("n,starts,samples,plain", [(64, 20, 250, False), (729, 20, 250, False), (729, 1, 69, False),
+                                                    (2744, 8, 200, False), (1728, 4, 100, True)])
+def test_large_biases_time_every_kernel(rules, dmax, n, starts, samples, plain):
+    """+-1 couplers past the byte-lane forms' biases: the warp-per-quad and the
+    streaming kernel are timed beside the integer quad groups."""
+    assert {STREAMING, WARP, INTEGER_QUADS} <= _kinds(rules, n, dmax=dmax, starts=starts, samples=samples, plain=plain)
+
+
+def test_problems_past_the_quad_groups_time_the_general_kernel(rules):
+    assert QUADS in _kinds(rules, 28200) and GENERAL not in _kinds(rules, 28200)
+    assert QUADS not in _kinds(rules, 28800) and GENERAL in _kinds(rules, 28800)
