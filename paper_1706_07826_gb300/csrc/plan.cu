@@ -445,14 +445,21 @@ std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin)
     const int blocks[3] = {128, 256, 512};
     const int qs[4] = {1, 2, 4, 8};
     const int quads = ceil_div(pl->C.S_fix, 4);
+    // small problems of any kind with many quads: the general kernel, whose items of 4 and 8 quads fill small
+    // blocks where a quad-group block's classes leave most of its threads idle (200 sweeps, 40 starts x (1000 +
+    // 1000): 8 spins, integer couplers 1.19 ms against 4.34, +-1 0.59 against 0.90; 27 spins 1.77 against 4.43;
+    // 64 spins, 20 x (250 + 250) 1.47 against 1.57; from 100 spins on it lost everywhere)
+    const bool small = pl->max_n0 < kGeneralSpins;
     for (int bi = 0; bi < 3; ++bi)
         for (int qi = 0; qi < 4; ++qi) {
             const int Q = qs[qi];
             if (Q > 1 && quads < Q) continue;
-            for (int stg = 1; others && stg >= 0; --stg) {
-                SweepShape sh{0, blocks[bi], Q, stg, 0, 0};
-                if (sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin) out.push_back(sh);
-            }
+            if (others || (small && bi < 2 && qi >= 2))
+                for (int stg = 1; stg >= (others ? 0 : 1); --stg) {
+                    SweepShape sh{0, blocks[bi], Q, stg, 0, 0};
+                    if (sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
+                        out.push_back(sh);
+                }
             if (pm1r_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
                 const int ns = plan_nslot(pl, Q, blocks[bi]);
                 const int md = pl->max_deg <= 6 ? 6 : 8;

@@ -519,6 +519,7 @@ struct PlanGeometry {
     uint64_t sig = 0;                 // structure signature of the problems (autotune cache key)
 };
 // Sweep shapes the autotuner times for a plan.
+constexpr int kGeneralSpins = 100;  // the general kernel is among them for problems of fewer spins
 std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin);
 
 // Everything one Multi-start SPVAR phase needs besides the slots.

@@ -103,3 +103,13 @@ def test_large_biases_time_every_kernel(rules, dmax, n, starts, samples, plain):
 def test_problems_past_the_quad_groups_time_the_general_kernel(rules):
     assert QUADS in _kinds(rules, 28200) and GENERAL not in _kinds(rules, 28200)
     assert QUADS not in _kinds(rules, 28800) and GENERAL in _kinds(rules, 28800)
+
+
+@pytest.mark.parametrize("pm1,jmax,dmax", [(True, 1, 12), (True, 1, 60), (False, 3, 30), (False, 90, 900)])
+@pytest.mark.parametrize("n", [8, 27, 64, 99])
+def test_small_problems_time_the_general_kernel(rules, n, pm1, jmax, dmax):
+    """A block of small problems' quads leaves most threads of a quad-group
+    block idle: the general kernel's items of 4 and 8 quads are timed too."""
+    out = rules("candidates", n, 2, 6, dmax, int(pm1), jmax, 20, 250, 0)
+    assert {"0:128:4", "0:128:8", "0:256:4", "0:256:8"} <= set(out)
+    assert GENERAL not in _kinds(rules, 100, dmax=dmax, pm1=pm1, jmax=jmax)
