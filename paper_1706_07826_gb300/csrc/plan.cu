@@ -516,13 +516,14 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
             return;
         }
     }
-    int Tt = std::min(pl->T, 128);
     // the trials run through the whole schedule in Tt sweeps, so that their reductions leave about as many
     // spins as the run's: on its first Tt rows (high temperatures) hardly a spin is fixed, and shapes that
-    // suit the full problem but not the small one of the solving phase won by up to 26 %
+    // suit the full problem but not the small one of the solving phase won by up to 33 %.  The simulated
+    // quantum annealing kernels read their own table row by row: their trials are its first Tt rows
+    int Tt = 0;
     auto set_sweeps = [&](int t) {
-        Tt = std::min(pl->T, t);
-        pl->trial_rows = std::max(1, pl->T / std::max(Tt, 1));
+        pl->trial_rows = pl->sqa_P > 0 ? 1 : trial_step(pl->T, t);
+        Tt = pl->sqa_P > 0 ? std::min(pl->T, t) : pl->T / pl->trial_rows;
     };
     set_sweeps(pl->sqa_P > 0 ? 64 : 128);
     int phases = 4;  // of a trial, at most

@@ -521,6 +521,9 @@ struct PlanGeometry {
 // Sweep shapes the autotuner times for a plan.
 constexpr int kGeneralSpins = 100;  // the general kernel is among them for problems of fewer spins
 std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin);
+// Rows of a schedule of T sweeps from one sweep of a trial of at most t to the next: the trial's T / step sweeps
+// reach to the schedule's end (all but less than one step of it).
+inline int trial_step(int T, int t) { return std::max(1, ceil_div(T, std::max(t, 1))); }
 
 // Everything one Multi-start SPVAR phase needs besides the slots.
 struct PhaseEngine {

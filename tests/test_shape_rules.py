@@ -49,6 +49,7 @@ int main(int argc, char **argv)
         g.sms = 152;
         for (const SweepShape &s : candidate_shapes(&g, kSmemOptin)) std::printf("%d:%d:%d ", s.kind, s.block, s.Q);
     }
+    if (!std::strcmp(argv[1], "trial")) std::printf("%d\n", trial_step(arg(2), arg(3)));
     return 0;
 }
 """
@@ -113,3 +114,12 @@ def test_small_problems_time_the_general_kernel(rules, n, pm1, jmax, dmax):
     out = rules("candidates", n, 2, 6, dmax, int(pm1), jmax, 20, 250, 0)
     assert {"0:128:4", "0:128:8", "0:256:4", "0:256:8"} <= set(out)
     assert GENERAL not in _kinds(rules, 100, dmax=dmax, pm1=pm1, jmax=jmax)
+
+
+@pytest.mark.parametrize("T", [0, 1, 100, 127, 128, 129, 200, 255, 256, 1000, 4097])
+@pytest.mark.parametrize("t", [128, 512])
+def test_trials_reach_the_schedules_end(rules, T, t):
+    step = int(rules("trial", T, t)[0])
+    sweeps = T // step
+    assert sweeps <= t and sweeps * step <= T       # no row past the table
+    assert T - sweeps * step < step                 # and the cold end is reached
