@@ -18,7 +18,6 @@
 #include <map>
 #include <mutex>
 #include <new>
-#include <tuple>
 #include <vector>
 
 #include "spvar_internal.h"
@@ -141,16 +140,7 @@ namespace {
 inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-struct TuneKey {
-    int max_n, max_deg, pm1, S, nslots, form, thr_stride, sqa_P;
-    uint64_t sig;
-    bool operator<(const TuneKey &o) const
-    {
-        return std::tie(max_n, max_deg, pm1, S, nslots, form, thr_stride, sqa_P, sig) <
-               std::tie(o.max_n, o.max_deg, o.pm1, o.S, o.nslots, o.form, o.thr_stride, o.sqa_P, o.sig);
-    }
-};
-std::map<TuneKey, SweepShape> g_tune_cache;
+std::map<std::vector<int64_t>, SweepShape> g_tune_cache;
 std::mutex g_tune_mu;
 
 void plan_free(spvar_plan *pl);
@@ -491,6 +481,16 @@ std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin)
     return out;
 }
 
+std::vector<int64_t> tune_key(const PlanGeometry *pl)
+{
+    auto octave = [](double x) { return (int64_t)std::floor(std::log2(std::max(x, 1e-9))); };
+    const spvar_params &p = pl->prm;
+    return {pl->max_n0, pl->max_deg, pl->pm1, pl->thr_stride, (int64_t)pl->sig, pl->C.nslots, p.form,
+            pl->C.S_fix, pl->C.S_solve, pl->C.S_corr, pl->sqa_P,
+            std::min<int64_t>(octave(pl->T), 12), std::min(pl->iters_max, 10), octave(p.elite_threshold),
+            octave(p.beta1), 16ll * p.fix_num / std::max(p.fix_den, 1), p.tree_preprocess, p.component_boost};
+}
+
 }  // namespace spvar
 
 namespace {
@@ -500,11 +500,10 @@ namespace {
 // millisecond, and four times as many of up to ten phases for the last choice;
 // the best of two repetitions after an untimed one, and one discarded trial
 // before the first candidate) for every candidate shape, the best four once
-// more, and keeps the fastest; results are cached per problem/plan geometry.
+// more, and keeps the fastest; results are cached by tune_key.
 void autotune(spvar_plan *pl, cudaStream_t st, int optin)
 {
-    const TuneKey key{pl->max_n0, pl->max_deg, pl->pm1 ? 1 : 0, pl->C.S_fix, pl->C.nslots,
-                      pl->prm.form, pl->thr_stride, pl->sqa_P, pl->sig};
+    const std::vector<int64_t> key = tune_key(pl);
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_tune_cache.find(key);

@@ -24,9 +24,10 @@ int main(int argc, char **argv)
         std::printf("%d %zu %d\n", (int)pm1q_request_ok(arg(2), arg(3), arg(4), arg(5), kSmemOptin), l.bytes + l.stat,
                     (int)l.tabs);
     }
-    if (!std::strcmp(argv[1], "candidates")) {
-        // spins, colour classes (of equal size), degree, dmax, +-1, largest coupler, starts, samples, plain form:
-        // kind and quads per item of every shape the autotuner times
+    if (!std::strcmp(argv[1], "candidates") || !std::strcmp(argv[1], "key")) {
+        // spins, colour classes (of equal size), degree, dmax, +-1, largest coupler, starts, samples, plain form,
+        // solving samples, sweeps, phases, elite in percent: the shapes the autotuner times, or the key they
+        // are kept by
         Problem P;
         std::memset(&P.hdr, 0, sizeof(P.hdr));
         P.hdr.n = arg(2);
@@ -36,7 +37,14 @@ int main(int argc, char **argv)
         PlanGeometry g;
         g.probs.push_back(&P);
         g.prm.form = arg(10) ? SPVAR_FORM_PLAIN : SPVAR_FORM_BATCHED;
-        g.C.S_fix = g.C.S_solve = g.C.Smax = arg(9);
+        g.C.S_fix = arg(9);
+        g.C.S_solve = argc > 11 ? arg(11) : arg(9);
+        g.C.Smax = std::max(g.C.S_fix, g.C.S_solve);
+        g.T = argc > 12 ? arg(12) : 1000;
+        g.iters_max = argc > 13 ? arg(13) : 2;
+        g.prm.elite_threshold = argc > 14 ? 0.01 * arg(14) : 0.1;
+        g.prm.beta1 = 3.0;
+        g.prm.fix_num = g.prm.fix_den = 1;
         g.C.nslots = arg(8);
         g.max_n0 = arg(2);
         g.max_deg = arg(4);
@@ -47,7 +55,10 @@ int main(int argc, char **argv)
         g.ncol_max = arg(3);
         g.class_max = P.csize[0];
         g.sms = 152;
-        for (const SweepShape &s : candidate_shapes(&g, kSmemOptin)) std::printf("%d:%d:%d ", s.kind, s.block, s.Q);
+        if (argv[1][0] == 'k')
+            for (int64_t x : tune_key(&g)) std::printf("%lld ", (long long)x);
+        else
+            for (const SweepShape &s : candidate_shapes(&g, kSmemOptin)) std::printf("%d:%d:%d ", s.kind, s.block, s.Q);
     }
     if (!std::strcmp(argv[1], "trial")) std::printf("%d\n", trial_step(arg(2), arg(3)));
     return 0;
@@ -123,3 +134,20 @@ def test_trials_reach_the_schedules_end(rules, T, t):
     sweeps = T // step
     assert sweeps <= t and sweeps * step <= T       # no row past the table
     assert T - sweeps * step < step                 # and the cold end is reached
+
+
+def test_plans_that_share_a_choice_have_the_same_candidates(rules):
+    """Two plans of one key are timed over the same shapes: the solving sample,
+    which decides whether few quads are launched, is part of it, and so is what
+    the trials depend on."""
+    seen = {}
+    for fixing, solving in ((50, 50), (50, 1000), (50, 0), (1000, 50)):
+        for starts in (1, 4, 40):
+            for T, phases, elite in ((100, 2, 10), (1000, 2, 10), (1000, 9, 10), (1000, 2, 50)):
+                a = (729, 2, 6, 12, 1, 1, starts, fixing, 0, solving, T, phases, elite)
+                key, shapes = tuple(rules("key", *a)), rules("candidates", *a)
+                assert key not in seen
+                seen[key] = shapes
+    base = (729, 2, 6, 12, 1, 1, 4, 100, 0, 100)
+    assert rules("key", *base, 1000, 2, 10) == rules("key", *base, 600, 2, 12)  # a scan's neighbours share it
+    assert rules("key", *base, 1000, 2, 10) != rules("key", *base, 400, 2, 10)
