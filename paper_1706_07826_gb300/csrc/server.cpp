@@ -113,11 +113,16 @@ struct spvar_server {
     // Size tiers: the same engine sized for max_n, max_n / 2, max_n / 4 and
     // max_n / 8 spins (shared memory per CTA, hence CTAs per SM, follow the size),
     // each with its persistent grid and captured phase graph; a step launches the
-    // smallest tier that holds every problem in flight.
-    struct Tier {
-        int max_n = 0, grid = 1;
+    // smallest tier that holds every problem in flight.  form[1], where the tier
+    // has one (grid > 0), is the streaming kernel for few quads in flight.
+    struct Form {
+        int grid = 0;
         PhaseEngine E{};
         cudaGraphExec_t graph = nullptr;
+    };
+    struct Tier {
+        int max_n = 0;
+        Form form[2];
     };
     std::vector<Tier> tiers;  // ascending max_n
     std::mutex mu;
@@ -306,19 +311,24 @@ int server_step(spvar_server *S, int32_t *active_out)
     if (!active) return SPVAR_OK;
     // the smallest size tier that holds every problem in flight
     int maxn = 0;
+    int64_t spins = 0;
     {
         std::lock_guard<std::mutex> g(S->mu);
         for (int64_t o : S->rslot_owner)
-            if (o >= 0) maxn = std::max(maxn, S->reqs[o]->hp.hdr.n);
+            if (o >= 0) {
+                maxn = std::max(maxn, S->reqs[o]->hp.hdr.n);
+                spins += S->reqs[o]->hp.hdr.n;
+            }
     }
     const spvar_server::Tier *tier = &S->tiers.back();
     for (const spvar_server::Tier &t : S->tiers)
         if (t.max_n >= maxn) { tier = &t; break; }
-    if (tier->graph) {
-        SPVAR_CUDA_TRY(cudaGraphLaunch(tier->graph, S->st));
+    const bool few = tier->form[1].grid > 0 && server_few_quads(spins * S->ns * ceil_div(S->Smax, 4), maxn, S->sms);
+    const spvar_server::Form &f = tier->form[few ? 1 : 0];
+    if (f.graph) {
+        SPVAR_CUDA_TRY(cudaGraphLaunch(f.graph, S->st));
     } else {
-        SPVAR_CUDA_TRY(engine_phase(tier->E, S->d_slots, S->nslots, S->cfg.params.num_sweeps, tier->grid, S->st,
-                                    false, false));
+        SPVAR_CUDA_TRY(engine_phase(f.E, S->d_slots, S->nslots, S->cfg.params.num_sweeps, f.grid, S->st, false, false));
     }
     SPVAR_CUDA_TRY(launch_gather_modes(S->d_slots, S->nslots, S->d_modes, S->st));
     SPVAR_CUDA_TRY(cudaMemcpyAsync(S->h_modes, S->d_modes, 4 * (size_t)S->nslots, cudaMemcpyDeviceToHost, S->st));
@@ -390,7 +400,8 @@ void server_free(spvar_server *S)
 {
     if (!S) return;
     for (spvar_server::Tier &t : S->tiers)
-        if (t.graph) cudaGraphExecDestroy(t.graph);
+        for (spvar_server::Form &f : t.form)
+            if (f.graph) cudaGraphExecDestroy(f.graph);
     if (S->cap_st) cudaStreamDestroy(S->cap_st);
     for (cudaEvent_t e : S->ev)
         if (e) cudaEventDestroy(e);
@@ -507,7 +518,8 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
     // items of Q quads of the largest admissible problem, more of smaller ones), else the
     // streaming +-1 kernel.  Measured at a request's 20 starts x (250 + 250) samples of 3D +-J
     // problems, quad-group against streaming: L = 9 6.4 against 13.2 ms, L = 12 10.8 against
-    // 14.0, L = 20 18.7 against 23.8.
+    // 14.0, L = 20 18.7 against 23.8.  With few quads in flight tiers whose groups hold four
+    // take the streaming kernel (server_few_quads).
     const int md = cfg->max_degree <= 6 ? 6 : 8;
     const bool pm1_only = p.sweep_kernel == SPVAR_SWEEP_PM1 || p.sweep_kernel == SPVAR_SWEEP_PM1S ||
                           p.sweep_kernel == SPVAR_SWEEP_PM1Q;
@@ -593,25 +605,35 @@ int spvar_server_create(const spvar_server_config *cfg, spvar_server **out)
         if (k > 0 && (tn < 256 || (!S->tiers.empty() && S->tiers.back().max_n == tn))) continue;
         spvar_server::Tier t;
         t.max_n = tn;
-        t.E = E;
-        t.E.max_n0 = tn;
-        t.E.C.max_n0 = tn;
-        if ((auto_quads || auto_gq) && !sqa) {
-            t.E.shape = auto_gq ? gq_default(tn, md, stride, (size_t)optin) : pm1q_default(tn, md, (size_t)optin);
-            t.E.C.Q = t.E.shape.Q;
+        SweepShape shapes[2] = {E.shape, SweepShape{-1, 0, 0, 0, 0, 0}};
+        if ((auto_quads || auto_gq) && !sqa)
+            shapes[0] = auto_gq ? gq_default(tn, md, stride, (size_t)optin) : pm1q_default(tn, md, (size_t)optin);
+        if (auto_quads && !sqa && pm1q_layout(shapes[0].block, tn, shapes[0].Q, md).nv > 1) {
+            const SweepShape sh{2, 512, 1, 0, 0, md};
+            if (pm1s_shape_ok(512, md, tn, 1) && sweep_shape_smem(sh, tn, stride, cfg->max_degree) <= (size_t)optin)
+                shapes[1] = sh;
         }
-        t.E.sweep_smem = sweep_shape_smem(t.E.shape, tn, stride, cfg->max_degree);
-        const int occ = std::max(1, sweep_shape_occupancy(t.E.shape, t.E.pm1, tn, stride, t.E.sweep_smem));
-        t.grid = occ * S->sms;
-        cudaGraph_t g = nullptr;
-        if (cudaStreamBeginCapture(S->cap_st, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
-            cudaError_t e = engine_phase(t.E, S->d_slots, S->nslots, T, t.grid, S->cap_st, false, true);
-            cudaError_t e2 = cudaStreamEndCapture(S->cap_st, &g);
-            if (e == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&t.graph, g, 0) != cudaSuccess)
-                t.graph = nullptr;
-            if (g) cudaGraphDestroy(g);
+        for (int v = 0; v < 2; ++v) {
+            if (shapes[v].kind < 0) continue;
+            spvar_server::Form &f = t.form[v];
+            f.E = E;
+            f.E.max_n0 = tn;
+            f.E.C.max_n0 = tn;
+            f.E.shape = shapes[v];
+            f.E.C.Q = f.E.shape.Q;
+            f.E.sweep_smem = sweep_shape_smem(f.E.shape, tn, stride, cfg->max_degree);
+            const int occ = std::max(1, sweep_shape_occupancy(f.E.shape, f.E.pm1, tn, stride, f.E.sweep_smem));
+            f.grid = occ * S->sms;
+            cudaGraph_t g = nullptr;
+            if (cudaStreamBeginCapture(S->cap_st, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
+                cudaError_t e = engine_phase(f.E, S->d_slots, S->nslots, T, f.grid, S->cap_st, false, true);
+                cudaError_t e2 = cudaStreamEndCapture(S->cap_st, &g);
+                if (e == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&f.graph, g, 0) != cudaSuccess)
+                    f.graph = nullptr;
+                if (g) cudaGraphDestroy(g);
+            }
+            cudaGetLastError();
         }
-        cudaGetLastError();
         S->tiers.push_back(t);
     }
     *out = S;

@@ -398,6 +398,11 @@ struct QuadLayout {
 };
 QuadLayout pm1q_layout(int block, int max_n, int Q, int maxd);
 SweepShape pm1q_default(int max_n, int maxd, size_t optin);
+// A server step of `load` spins times quads, the largest problem of maxn spins, takes the streaming kernel instead of
+// groups of four quads, which are at least one item's work however few there are: up to three quads of the largest
+// size per SM.  300 sweeps, streaming against quad groups: two requests of 13 quads, L = 12, 1.84 and 4.21 ms; of 100
+// 3.94 and 5.49; of 200 (L = 6) 1.71 and 1.94; beyond, two of 400, L = 12, 7.13 and 5.97, L = 9 7.24 and 4.17.
+inline bool server_few_quads(long long load, int maxn, int sms) { return load <= 3ll * sms * maxn; }
 // The kernel exists and its static and dynamic shared memory fit a CTA.
 bool pm1q_fits(int block, int max_n, int Q, int maxd, size_t optin);
 // A requested item of Q quads is taken where two copies of every quad's spin words, and the launch itself, fit a CTA.

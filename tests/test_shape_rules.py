@@ -60,6 +60,7 @@ int main(int argc, char **argv)
         else
             for (const SweepShape &s : candidate_shapes(&g, kSmemOptin)) std::printf("%d:%d:%d ", s.kind, s.block, s.Q);
     }
+    if (!std::strcmp(argv[1], "few")) std::printf("%d\n", (int)server_few_quads(std::atoll(argv[2]), arg(3), arg(4)));
     if (!std::strcmp(argv[1], "trial")) std::printf("%d\n", trial_step(arg(2), arg(3)));
     return 0;
 }
@@ -151,3 +152,11 @@ def test_plans_that_share_a_choice_have_the_same_candidates(rules):
     base = (729, 2, 6, 12, 1, 1, 4, 100, 0, 100)
     assert rules("key", *base, 1000, 2, 10) == rules("key", *base, 600, 2, 12)  # a scan's neighbours share it
     assert rules("key", *base, 1000, 2, 10) != rules("key", *base, 400, 2, 10)
+
+
+def test_server_steps_of_few_quads(rules):
+    """Three quads of the largest problem in flight per SM, smaller problems by their spins."""
+    for quads, n, few in ((26, 1728, 1), (456, 216, 1), (457, 216, 0), (800, 729, 0)):
+        assert int(rules("few", quads * n, n, 152)[0]) == few
+    assert int(rules("few", 400 * 64 + 400 * 1728, 1728, 152)[0]) == 1
+    assert int(rules("few", 16384 * 4096 * 32768, 32768, 152)[0]) == 0  # past 32 bits
