@@ -787,10 +787,17 @@ int spvar_reduce(const spvar_problem *p, const int8_t *fixed, int32_t *old_of_ne
     Problem *D = new (std::nothrow) Problem();
     if (!D) return SPVAR_ENOMEM;
     D->device = S->device;
-    // one allocation: the fold's scratch behind the problem's arrays
-    const size_t prob_bytes = prob_blob_bytes(H.cap_n, H.cap_nnz, H.maxdeg);
-    D->blob_bytes = prob_bytes + 4 * slot_scratch_ints(H.cap_n);
+    D->blob_bytes = prob_blob_bytes(H.cap_n, H.cap_nnz, H.maxdeg);
+    // the fold's scratch is freed at the call's end: behind the problem's arrays it saved an allocation (2 of 78 us
+    // at 8000 spins) and stayed with the handle, 12 bytes a spin and 20 KB
+    int32_t *scratch = nullptr;
     if (cudaMalloc(&D->blob, D->blob_bytes) != cudaSuccess) {
+        delete D;
+        cudaGetLastError();
+        return SPVAR_ENOMEM;
+    }
+    if (cudaMalloc(&scratch, 4 * slot_scratch_ints(H.cap_n)) != cudaSuccess) {
+        cudaFree(D->blob);
         delete D;
         cudaGetLastError();
         return SPVAR_ENOMEM;
@@ -798,7 +805,6 @@ int spvar_reduce(const spvar_problem *p, const int8_t *fixed, int32_t *old_of_ne
     std::memset(&D->hdr, 0, sizeof(DevProb));
     prob_carve(&D->hdr, D->blob, H.cap_n, H.cap_nnz, H.maxdeg);
     D->dev = static_cast<DevProb *>(D->blob);
-    int32_t *scratch = reinterpret_cast<int32_t *>(static_cast<char *>(D->blob) + prob_bytes);
     cudaStream_t st = as_stream(stream);
     bool ok = launch_reduce_single(S->dev, D->dev, D->hdr, fixed, old_of_new, scratch, st) == cudaSuccess;
     DevProb back;
@@ -806,6 +812,7 @@ int spvar_reduce(const spvar_problem *p, const int8_t *fixed, int32_t *old_of_ne
     if (ok) ok = cudaMemcpyAsync(&back, D->dev, sizeof(DevProb), cudaMemcpyDeviceToHost, st) == cudaSuccess;
     if (ok) ok = cudaMemcpyAsync(cptr, D->hdr.cptr, sizeof(cptr), cudaMemcpyDeviceToHost, st) == cudaSuccess;
     if (ok) ok = cudaStreamSynchronize(st) == cudaSuccess;
+    cudaFree(scratch);
     if (!ok) {
         cudaFree(D->blob);
         delete D;

@@ -996,7 +996,7 @@ __device__ __forceinline__ void fold_cluster(Slot &s, int n, int rank)
 // The standalone reduction: the pass's fold stages on one cluster.  Bound by
 // the latency of its dependent gathers, which one CTA of 1024 threads walked
 // through a spin at a time: 64 us of device time at 8000 spins, about 20 here
-// (the call 150.8 -> 78.7 us, with one allocation and one wait less).
+// (the call 150.8 -> 80 us, with one wait less).
 __global__ void __cluster_dims__(kPassCluster, 1, 1) __launch_bounds__(kPassBlock)
     k_reduce_single(const DevProb *src, DevProb *dst, DevProb hdr, const int8_t *fixed,
                     int32_t *old_of_new, int32_t *scratch)
