@@ -502,17 +502,19 @@ __device__ void run_item_sqa(const SweepLaunch &L, const SweepJob &job, int quad
 // Chimera C8, 10 starts x (500 + 500), 16 slices, 500 sweeps: 46.5 ms with two CTAs and
 // carries of u + entry, 44.6 ms with three, one comparison per replica and the row's
 // address merged by the byte permute; the two integer pipes bound it (18 wide multiplies
-// and about 50 ALU instructions per four-replica item).
-template <int B, int MAXD, int NC, bool SI>
+// and about 50 ALU instructions per four-replica item).  FEW: a launch of at most two blocks an SM, which
+// the registers of the third would only cost: 3D L = 4, 4 slices, 100 sweeps, 180 blocks 0.349 ms with two
+// asked for and carries, 0.360 with three, 0.335 with two.
+template <int B, int MAXD, int NC, bool SI, bool FEW>
 constexpr int sqa_min_blocks()
 {
-    return NC > 0 && B == 256 ? (NC == 2 && !SI && MAXD == 6 ? 3 : 2) : 1;
+    return NC > 0 && B == 256 ? (NC == 2 && !SI && MAXD == 6 && !FEW ? 3 : 2) : 1;
 }
 
 // NC > 0: register form for problems of at most NC colour classes of at most
 // B spins (+-1 or small integer couplers, two or more slices); 0: the item walk.
-template <bool PM1, int B, int MAXD, int NC, int E, bool SI>
-__global__ void __launch_bounds__(B, sqa_min_blocks<B, MAXD, NC, SI>()) k_sweep_sqa(const SweepLaunch L)
+template <bool PM1, int B, int MAXD, int NC, int E, bool SI, bool FEW = false>
+__global__ void __launch_bounds__(B, sqa_min_blocks<B, MAXD, NC, SI, FEW>()) k_sweep_sqa(const SweepLaunch L)
 {
     extern __shared__ __align__(16) uint32_t smem_sqa[];
     __shared__ SqaStatic<(NC > 0)> sm;
@@ -572,6 +574,15 @@ void *select_sqa(int variant, int block, int maxdeg, int ncls, int e)
     return nullptr;
 }
 
+// The same for a launch of at most two blocks an SM, where that is another kernel, else null.
+void *select_sqa_few(int variant, int block, int maxdeg, int ncls, int e)
+{
+    if (variant != 2 || block != 256 || maxdeg > 6 || ncls != 2) return nullptr;
+    return e == 2   ? reinterpret_cast<void *>(k_sweep_sqa<true, 256, 6, 2, 2, false, true>)
+           : e == 1 ? reinterpret_cast<void *>(k_sweep_sqa<true, 256, 6, 2, 1, false, true>)
+                    : reinterpret_cast<void *>(k_sweep_sqa<true, 256, 6, 2, 0, false, true>);
+}
+
 // Form of the acceptance rows (see sqa_reg_items).
 int sqa_entries(bool ent32, int W) { return !ent32 ? 0 : 3 * W <= 64 ? 2 : 1; }
 
@@ -599,6 +610,11 @@ cudaError_t launch_sweep_sqa(const SweepLaunch &L, int variant, int block, int n
 {
     void *k = select_sqa(variant, block, L.max_deg, ncls, sqa_entries(ent32, L.W));
     if (!k) return cudaErrorInvalidValue;
+    void *few = select_sqa_few(variant, block, L.max_deg, ncls, sqa_entries(ent32, L.W));
+    int dev = 0, sms = 0;
+    if (few && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && grid <= 2 * sms)
+        k = few;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<SweepLaunch *>(&L)};
