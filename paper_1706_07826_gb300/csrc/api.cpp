@@ -351,6 +351,9 @@ SweepShape register_shape(const Problem *P, int quads, int sms, int optin, int t
     // Where large classes leave many threads of every slot over, and with several items per SM, the
     // quad-group kernel is the faster one (Chimera C9, 324 spins a class in two slots of 256: 8000
     // samples, 400 sweeps, 2885 -> 2536 us; 10000 samples, a last round of items nearly empty, stay).
+    // Its rounds take 0.154 n ns from 512 spins on; below, an item's fixed part decides, the estimate is
+    // too low (3D L = 3 .. 6 chosen by it ran 2 to 5 times slower) and the comparison is not made.  Both
+    // estimates are good to about 10 %, hence 0.88.
     if (mode == 0 && best.block > 0 && quads >= 6 * sms && P->hdr.n >= 512) {
         double rounds = 0.0;
         const SweepShape g = quad_group_shape(P, quads, sms, optin, thr_stride, true, &rounds);

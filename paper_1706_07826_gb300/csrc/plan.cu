@@ -495,8 +495,8 @@ std::vector<int64_t> tune_key(const PlanGeometry *pl)
 
 namespace {
 
-// Times a short run of the plan's phases (at most 4, 128 sweeps each that step
-// through the whole schedule, up to 512 where a trial is shorter than a
+// Times a short run of the plan's phases (at most 4, about 128 sweeps each that step
+// through the whole schedule, up to about 512 where a trial is shorter than a
 // millisecond, and four times as many of up to ten phases for the last choice;
 // the best of two repetitions after an untimed one, and one discarded trial
 // before the first candidate) for every candidate shape, the best four once

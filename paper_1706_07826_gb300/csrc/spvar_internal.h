@@ -530,9 +530,9 @@ std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin);
 // the trials go.  Sample sizes enter as they are; the schedule's length, the elite and the final inverse
 // temperature by octaves, so that a scan over them does not pay for trials (0.1 to 0.5 s) at every value.
 std::vector<int64_t> tune_key(const PlanGeometry *pl);
-// Rows of a schedule of T sweeps from one sweep of a trial of at most t to the next: the trial's T / step sweeps
-// reach to the schedule's end (all but less than one step of it).
-inline int trial_step(int T, int t) { return std::max(1, ceil_div(T, std::max(t, 1))); }
+// Rows of a schedule of T sweeps from one sweep of a trial of about t to the next: the trial's T / step sweeps, t to
+// 2 t of them (or all), reach to the schedule's end but for less than one step.
+inline int trial_step(int T, int t) { return std::max(1, T / std::max(t, 1)); }
 
 // Everything one Multi-start SPVAR phase needs besides the slots.
 struct PhaseEngine {
