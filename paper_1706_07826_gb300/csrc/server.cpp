@@ -224,6 +224,8 @@ int place_request(spvar_server *S, Request &R)
     C.nslots = S->ns;
     if (ok) ok = launch_slots_init(d, C, n0, S->st) == cudaSuccess;
     if (ok) ok = cudaStreamSynchronize(S->st) == cudaSuccess;
+    for (int k = 0; k < S->ns; ++k)
+        S->h_modes[(size_t)R.rslot * S->ns + k] = (C.S_corr > 0 && hp.hdr.hzero) ? kCorr : kFixing;
     return ok ? SPVAR_OK : SPVAR_ECUDA;
 }
 
@@ -311,19 +313,23 @@ int server_step(spvar_server *S, int32_t *active_out)
     if (!active) return SPVAR_OK;
     // the smallest size tier that holds every problem in flight
     int maxn = 0;
-    int64_t spins = 0;
+    int64_t load = 0;  // spins times quads of the phases the starts are in
     {
         std::lock_guard<std::mutex> g(S->mu);
-        for (int64_t o : S->rslot_owner)
-            if (o >= 0) {
-                maxn = std::max(maxn, S->reqs[o]->hp.hdr.n);
-                spins += S->reqs[o]->hp.hdr.n;
+        for (size_t r = 0; r < S->rslot_owner.size(); ++r) {
+            if (S->rslot_owner[r] < 0) continue;
+            const int n = S->reqs[S->rslot_owner[r]]->hp.hdr.n;
+            maxn = std::max(maxn, n);
+            for (int k = 0; k < S->ns; ++k) {
+                const int mode = S->h_modes[r * S->ns + k];
+                if (mode != kDone) load += (int64_t)n * ceil_div(phase_samples(S->E.C, mode), 4);
             }
+        }
     }
     const spvar_server::Tier *tier = &S->tiers.back();
     for (const spvar_server::Tier &t : S->tiers)
         if (t.max_n >= maxn) { tier = &t; break; }
-    const bool few = tier->form[1].grid > 0 && server_few_quads(spins * S->ns * ceil_div(S->Smax, 4), maxn, S->sms);
+    const bool few = tier->form[1].grid > 0 && server_few_quads(load, maxn, S->sms);
     const spvar_server::Form &f = tier->form[few ? 1 : 0];
     if (f.graph) {
         SPVAR_CUDA_TRY(cudaGraphLaunch(f.graph, S->st));
