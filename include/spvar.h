@@ -478,9 +478,9 @@ typedef struct spvar_server spvar_server;
 
 typedef struct spvar_server_config {
     spvar_params params;    /* Alg. 2 parameters of every request; sweep_kernel = SPVAR_SWEEP_PM1
-                               restricts the server to +-1 couplers (the quad-group kernel, or with a
-                               block or replica count given the streaming one; SPVAR_SWEEP_PM1Q: the
-                               quad-group kernel) */
+                               restricts the server to +-1 couplers (the quad-group kernel, the
+                               streaming one while few quads are in flight or with a block or replica
+                               count given; SPVAR_SWEEP_PM1Q: the quad-group kernel where it fits) */
     size_t budget_bytes;    /* device memory for admitted requests' workspaces */
     int32_t max_n;          /* largest request: spins, CSR entries, degree */
     int32_t max_nnz;

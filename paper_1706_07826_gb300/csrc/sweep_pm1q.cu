@@ -23,7 +23,8 @@
 // keys kept in registers, the row's address merged by the byte permute that extracts
 // the index, one comparison per replica).  3D +-J batch, 64 problems of L = 6 .. 12,
 // 2000 + 2000 samples, 1000 sweeps: 271 ms with one quad per word and no records,
-// 174 ms now (1.2e12 attempts/s).
+// 175 ms now (1.2e12 attempts/s).  Two pairs a group need more than the 64 registers
+// of two 512-thread blocks an SM: those forms spill 20 to 72 bytes (the batch's 32).
 // Eligible when every |J| = 1, degree <= MAXD <= 8 and dmax <= 30.
 #include "quad_units.cuh"
 

@@ -32,7 +32,8 @@
 // a queue search per temperature, 28.9 ms now (3.4e11 Metropolis attempts/s).  Of a
 // sweep's time the Metropolis part takes 25 us (150 instructions per four attempts of 32
 // lanes, Philox 70 of them), the cluster moves 20 us (82 us with the queue search: 500
-// instructions a step), the exchanges 4 us and the kept lists 7 us.
+// instructions a step), the exchanges 4 us and the kept lists 7 us.  The byte-lane forms
+// spill 52 to 92 bytes at the 64 registers of two CTAs an SM.
 #include <climits>
 #include <cstring>
 
