@@ -248,7 +248,7 @@ int host_problem_upload(const HostProblem &hp, void *blob, cudaStream_t st, DevP
 
 }  // namespace spvar
 
-namespace {
+namespace spvar {
 
 // Shape of one sample of `quads` quads on a quad-group kernel (pm1: +-1 couplers, else integer
 // ones): block size and quads per item whose busiest SM is done first.  A thread's work per
@@ -260,14 +260,14 @@ namespace {
 // 12 with 250 quads 1.43 ms (1024 threads, pairs) against 1.69 streaming, with 100 quads
 // 1.13 against 0.98 streaming; L = 9 with 50 quads 1.09 against 1.35 streaming.
 // *cost (if not null): the busiest SM's rounds per sweep, one of which takes about 0.15 n ns.
-SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, bool pm1,
-                            double *cost = nullptr)
+SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, bool pm1, double *cost)
 {
     const DevProb &H = P->hdr;
     const int md = H.maxdeg <= 6 ? 6 : 8;
     SweepShape best{pm1 ? 6 : 7, 0, 1, 0, 0, md};
     double best_t = 1e300;
-    for (int B : {512, 1024})
+    for (int B : {512, 1024}) {
+        int qb = 0;  // quads per item of this block's best so far
         for (int Q : {1, 2, 4, 8, 16}) {
             // 16 quads of integer couplers only where 8 leave a second round of items, two blocks an SM: small
             // problems fill no block with 8 (200 sweeps, 16000 samples, 6 spins: 0.70 ms in two rounds, against
@@ -297,12 +297,16 @@ SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int
                 work += std::min(all, ceil(nc * groups / B) * (0.4 + len));
             }
             const double t = ceil((double)k / conc) * work * std::max(conc * B / 128.0, 4.0);
-            if (t <= best_t) {
+            // equal estimates: the larger block (its rounds are fewer), and more quads an item only where fewer leave
+            // some SM a second one, since units that fill a block's idle warps are not free (degree 8, |J| <= 39, 200
+            // spins, 10 quads, 50 sweeps: 0.187 ms as two items of 8, 0.147 on the general kernel, 0.106 as ten of one)
+            if (t < best_t || (t == best_t && (qb == 0 || ceil_div(quads, qb) > sms))) {
                 best_t = t;
                 best.block = B;
-                best.Q = Q;
+                best.Q = qb = Q;
             }
         }
+    }
     if (cost) *cost = best_t;
     if (pm1 && best.block > 0 && pm1s_shape_ok(512, md, H.n, 1)) {
         const int bytes = (int)pm1s_smem_bytes(H.n, 1, md) + (2 << 10), k = ceil_div(quads, sms);
@@ -313,6 +317,10 @@ SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int
     }
     return best;
 }
+
+}  // namespace spvar
+
+namespace {
 
 // Shape of one sample of `quads` quads on the register kernel (mode 0: byte lanes, 1 and 2: the
 // 16-bit lanes): the block size and quads per item whose busiest SM is done first.  A slot (a

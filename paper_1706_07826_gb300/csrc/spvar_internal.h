@@ -508,6 +508,10 @@ inline int sweep_shape_occupancy(const SweepShape &s, bool pm1, int max_n, int t
     return sweep_max_active_blocks(pm1, s.block, smem, s.stage != 0);
 }
 
+// Shape of one sample on a quad-group kernel (or, few quads of a large +-1 problem, the streaming one).
+SweepShape quad_group_shape(const Problem *P, int quads, int sms, int optin, int thr_stride, bool pm1,
+                            double *cost = nullptr);
+
 // What the choice of a plan's sweep shape depends on.
 struct PlanGeometry {
     std::vector<const Problem *> probs;

@@ -24,16 +24,22 @@ int main(int argc, char **argv)
         std::printf("%d %zu %d\n", (int)pm1q_request_ok(arg(2), arg(3), arg(4), arg(5), kSmemOptin), l.bytes + l.stat,
                     (int)l.tabs);
     }
-    if (!std::strcmp(argv[1], "candidates") || !std::strcmp(argv[1], "key")) {
+    if (!std::strcmp(argv[1], "candidates") || !std::strcmp(argv[1], "key") || !std::strcmp(argv[1], "sample")) {
         // spins, colour classes (of equal size), degree, dmax, +-1, largest coupler, starts, samples, plain form,
-        // solving samples, sweeps, phases, elite in percent: the shapes the autotuner times, or the key they
-        // are kept by
+        // solving samples, sweeps, phases, elite in percent: the shapes the autotuner times, the key they are
+        // kept by, or the quad-group shape of one sample
         Problem P;
         std::memset(&P.hdr, 0, sizeof(P.hdr));
         P.hdr.n = arg(2);
         P.hdr.ncol = arg(3);
         for (int c = 0; c < arg(3); ++c) P.csize[c] = arg(2) / arg(3) + (c < arg(2) % arg(3));
         P.jabs_max = arg(7);
+        if (argv[1][0] == 's') {
+            P.hdr.maxdeg = arg(4);
+            const SweepShape s = quad_group_shape(&P, (arg(9) + 3) / 4, 152, kSmemOptin, arg(5) + 1, arg(6) != 0);
+            std::printf("%d:%d:%d\n", s.kind, s.block, s.Q);
+            return 0;
+        }
         PlanGeometry g;
         g.probs.push_back(&P);
         g.prm.form = arg(10) ? SPVAR_FORM_PLAIN : SPVAR_FORM_BATCHED;
@@ -160,3 +166,13 @@ def test_server_steps_of_few_quads(rules):
         assert int(rules("few", quads * n, n, 152)[0]) == few
     assert int(rules("few", 400 * 64 + 400 * 1728, 1728, 152)[0]) == 1
     assert int(rules("few", 16384 * 4096 * 32768, 32768, 152)[0]) == 0  # past 32 bits
+
+
+@pytest.mark.parametrize("n,ncol,deg,dmax,samples,quads", [
+    (200, 4, 8, 472, 40, 1),        # ten items of one quad, not two of eight whose units fill idle warps
+    (200, 4, 8, 472, 600, 1),
+    (27, 3, 6, 900, 16000, 16),     # one round of 250 items, not two of 500
+    (27, 3, 6, 900, 9728, 8)])
+def test_quads_per_item_of_an_integer_sample(rules, n, ncol, deg, dmax, samples, quads):
+    kind, block, q = rules("sample", n, ncol, deg, dmax, 0, 40, 1, samples, 0)[0].split(":")
+    assert (int(kind), int(q)) == (INTEGER_QUADS, quads)
