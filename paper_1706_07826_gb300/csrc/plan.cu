@@ -416,16 +416,23 @@ std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin)
     // +-1 couplers with large biases (dmax 31 .. 254): a warp per quad, and the streaming kernel (200 sweeps,
     // dmax 32: L = 9, 20 starts x (250 + 250) 2.52 ms warp per quad, 3.34 the integer quad groups; L = 4 0.65
     // and 0.74; L = 14, 8 starts x (200 + 200), four phases 3.99 ms streaming and 4.20)
-    if ((others || !quads_ok) && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
+    // With smaller biases a warp per quad only for problems of more than four colour classes, which the register
+    // kernel's slots do not hold, or of fewer than 512 spins: small or uneven classes close with a warp's own barrier
+    // (random degree 8, 20 spins, 20 starts x (114 + 114), four phases, 150 sweeps: 0.71 ms against 0.76; degree 6,
+    // 286 spins, 24 x (254 + 254), 300 sweeps 5.6 against 6.0)
+    const bool uneven = quads_ok && (pl->ncol_max > 4 || pl->max_n0 < 512);
+    if ((others || !quads_ok || uneven) && pm1_kernel_eligible(pl->pm1, pl->dmax, pl->max_deg)) {
         const int md = pl->max_deg <= 6 ? 6 : 8;
         for (int w : {2, 4, 8, 16})
             for (int K : {2, 4}) {
+                if (quads_ok && !others && w > 4) continue;
                 SweepShape sh{4, 32 * w, w, 0, K, md};
                 if (pm1w_shape_ok(w, md, pl->max_n0, K) &&
                     sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
                     out.push_back(sh);
             }
         for (int b : {128, 256, 512, 1024}) {
+            if (quads_ok && !others) break;
             SweepShape sh{2, b, 1, 0, 0, md};
             if (pm1s_shape_ok(b, md, pl->max_n0, 1) &&
                 sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)
@@ -438,13 +445,14 @@ std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin)
     // small problems of any kind with many quads: the general kernel, whose items of 4 and 8 quads fill small
     // blocks where a quad-group block's classes leave most of its threads idle (200 sweeps, 40 starts x (1000 +
     // 1000): 8 spins, integer couplers 1.19 ms against 4.34, +-1 0.59 against 0.90; 27 spins 1.77 against 4.43;
-    // 64 spins, 20 x (250 + 250) 1.47 against 1.57; from 100 spins on it lost everywhere)
+    // 64 spins, 20 x (250 + 250) 1.47 against 1.57; with uneven classes, random degree 6, 100 spins, 13 x (850 +
+    // 850), 60 sweeps 1.01 against 1.16; from 160 spins on it lost everywhere)
     const bool small = pl->max_n0 < kGeneralSpins;
     for (int bi = 0; bi < 3; ++bi)
         for (int qi = 0; qi < 4; ++qi) {
             const int Q = qs[qi];
             if (Q > 1 && quads < Q) continue;
-            if (others || (small && bi < 2 && qi >= 2))
+            if (others || (small && qi >= 2))
                 for (int stg = 1; stg >= (others ? 0 : 1); --stg) {
                     SweepShape sh{0, blocks[bi], Q, stg, 0, 0};
                     if (sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg) <= (size_t)optin)

@@ -528,7 +528,7 @@ struct PlanGeometry {
     uint64_t sig = 0;                 // structure signature of the problems (autotune cache key)
 };
 // Sweep shapes the autotuner times for a plan.
-constexpr int kGeneralSpins = 100;  // the general kernel is among them for problems of fewer spins
+constexpr int kGeneralSpins = 192;  // the general kernel is among them for problems of fewer spins
 std::vector<SweepShape> candidate_shapes(const PlanGeometry *pl, int optin);
 // Plans of one key share the autotuner's choice: everything the candidates depend on, and what decides how
 // the trials go.  Sample sizes enter as they are; the schedule's length, the elite and the final inverse

@@ -125,13 +125,13 @@ def test_problems_past_the_quad_groups_time_the_general_kernel(rules):
 
 
 @pytest.mark.parametrize("pm1,jmax,dmax", [(True, 1, 12), (True, 1, 60), (False, 3, 30), (False, 90, 900)])
-@pytest.mark.parametrize("n", [8, 27, 64, 99])
+@pytest.mark.parametrize("n", [8, 27, 64, 191])
 def test_small_problems_time_the_general_kernel(rules, n, pm1, jmax, dmax):
     """A block of small problems' quads leaves most threads of a quad-group
     block idle: the general kernel's items of 4 and 8 quads are timed too."""
     out = rules("candidates", n, 2, 6, dmax, int(pm1), jmax, 20, 250, 0)
-    assert {"0:128:4", "0:128:8", "0:256:4", "0:256:8"} <= set(out)
-    assert GENERAL not in _kinds(rules, 100, dmax=dmax, pm1=pm1, jmax=jmax)
+    assert {"0:128:4", "0:128:8", "0:256:4", "0:256:8", "0:512:4", "0:512:8"} <= set(out)
+    assert GENERAL not in _kinds(rules, 192, dmax=dmax, pm1=pm1, jmax=jmax)
 
 
 @pytest.mark.parametrize("T", [0, 1, 100, 127, 128, 129, 200, 255, 256, 1000, 4097])
@@ -176,3 +176,11 @@ def test_server_steps_of_few_quads(rules):
 def test_quads_per_item_of_an_integer_sample(rules, n, ncol, deg, dmax, samples, quads):
     kind, block, q = rules("sample", n, ncol, deg, dmax, 0, 40, 1, samples, 0)[0].split(":")
     assert (int(kind), int(q)) == (INTEGER_QUADS, quads)
+
+
+def test_small_and_many_classes_time_a_warp_per_quad(rules):
+    """Past four classes the register kernel has no slots for a +-1 problem, and
+    small classes leave a quad-group block's threads idle."""
+    for n, ncol in ((20, 5), (83, 8), (286, 4), (511, 2), (2000, 5)):
+        assert WARP in _kinds(rules, n, deg=8, dmax=18, ncol=ncol)
+    assert WARP not in _kinds(rules, 512, deg=8, dmax=18, ncol=4)
