@@ -540,26 +540,38 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
+    const bool plain = pl->prm.form == SPVAR_FORM_PLAIN;
+    const int trial_slots = plain ? 1 : pl->C.nslots;
+    // makes sh the plan's shape; its grid in a trial (0: it does not launch)
+    auto set_shape = [&](const SweepShape &sh) -> int {
+        pl->shape = sh;
+        pl->sweep_smem = sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg);
+        if (sweep_shape_occupancy(sh, pl->pm1, pl->max_n0, pl->thr_stride, pl->sweep_smem) < 1) return 0;
+        const int items = trial_slots * ceil_div(ceil_div(pl->C.Smax, 4), sh.Q);
+        return plain ? items : grid_for(pl, items);
+    };
+    // every shape that launches, and the balanced form where its grid is another
     std::vector<SweepShape> cands;
     for (SweepShape sh : candidate_shapes(pl, optin)) {
+        const int full = set_shape(sh);
+        if (full < 1) {
+            cudaGetLastError();
+            continue;
+        }
         cands.push_back(sh);
         sh.balance = 1;
-        if (pl->prm.form != SPVAR_FORM_PLAIN) cands.push_back(sh);
+        if (!plain && set_shape(sh) != full) cands.push_back(sh);
     }
     // a short run of the plan's phases (fixing, and solving on the problems it
     // reduced), so that shapes that suit the full problem but not the reduced
     // ones are not picked; chunk_t > 0 splits every phase into sweep launches
-    auto trial = [&](const SweepShape &sh, int chunk_t) -> float {
-        pl->shape = sh;
-        pl->sweep_smem = sweep_shape_smem(sh, pl->max_n0, pl->thr_stride, pl->max_deg);
-        if (sweep_shape_occupancy(sh, pl->pm1, pl->max_n0, pl->thr_stride, pl->sweep_smem) < 1) return 1e30f;
-        const int nslots = (pl->prm.form == SPVAR_FORM_PLAIN) ? 1 : pl->C.nslots;
+    // (a shape a quarter slower than `bound` is not repeated)
+    auto trial = [&](const SweepShape &sh, int chunk_t, float bound = 1e30f) -> float {
+        const int nslots = trial_slots, grid = set_shape(sh);
         pl->C.Q = sh.Q;
         pl->C.chunk = chunk_t;
         SolveConsts C = pl->C;
         C.nslots = nslots;
-        const int items = nslots * ceil_div(ceil_div(pl->C.Smax, 4), sh.Q);
-        const int grid = (pl->prm.form == SPVAR_FORM_PLAIN) ? items : grid_for(pl, items);
         const int launches = std::min(pl->iters_max, phases) * launches_per_phase(Tt, chunk_t);
         float ms = 1e30f;
         bool ok = true;
@@ -573,6 +585,7 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
             float m = 0.f;
             cudaEventElapsedTime(&m, a, b);
             if (rep > 0) ms = std::min(ms, m);  // the first repetition includes one-time setup
+            if (ms < 1e30f && ms > 1.25f * bound) break;
         }
         pl->C.chunk = 0;
         if (!ok) { cudaGetLastError(); return 1e30f; }
@@ -586,9 +599,11 @@ void autotune(spvar_plan *pl, cudaStream_t st, int optin)
         if (ms < 1.0f && pl->sqa_P == 0) set_sweeps(128 * std::min(4, (int)(1.0f / std::max(ms, 0.1f)) + 1));
     }
     std::vector<std::pair<float, size_t>> times;
+    float least = 1e30f;
     for (size_t i = 0; i < cands.size(); ++i) {
-        const float ms = trial(cands[i], 0);
+        const float ms = trial(cands[i], 0, least);
         if (ms < 1e30f) times.emplace_back(ms, i);
+        least = std::min(least, ms);
     }
     // the candidates within 5 % of the best, at most four, once more, and where that takes a few
     // milliseconds at four times the sweeps, whose reductions are nearer to the run's: single short
